@@ -50,19 +50,6 @@ __device__ __forceinline__ int key_row(const unsigned long long *tab, uint32_t m
     return -1;
 }
 
-// Set of (in << 24 | out) pairs.  True when the pair was already present.
-__device__ __forceinline__ bool pair_insert(unsigned long long *tab, uint32_t mask, unsigned long long pair)
-{
-    uint32_t s = tslot(pair, mask);
-    for (uint32_t probe = 0; probe <= mask; ++probe) {
-        const unsigned long long old = atomicCAS(tab + s, kFree, pair);
-        if (old == kFree) return false;
-        if (old == pair) return true;
-        s = (s + 1u) & mask;
-    }
-    return false;
-}
-
 // (in << 24 | out) pair -> lowest row holding it (entries pair << 13 | row,
 // row < 8192).
 __device__ __forceinline__ void pair_row_insert(unsigned long long *tab, uint32_t mask, unsigned long long pair,
