@@ -7,14 +7,31 @@
 // of [-1,1]^2, node index = res * iy + ix.  Output layout
 // weights[genome][block][source][target], block l joining layer l to l+1.
 //
-// GB300 mapping: a block of 256 threads takes (genome, chunk of queries),
-// bulk-copies the genome's record into shared memory once (TMA + mbarrier),
-// and each thread evaluates its own queries one after another in its own
-// column of the value tile v[position][256]: node and edge reads are the same
-// for the whole warp (broadcasts), value reads hit 32 distinct banks, and no
-// barrier is needed between nodes.  The work is bound by FP32 and SFU issue
-// (edges and transcendentals per query), not by memory: the only traffic is
-// the 4-byte output per query.
+// Every block of the weights has the same value for the same (source, target)
+// pair: the layers share one grid and a query holds no layer coordinate.  Each
+// pair is evaluated once and its weight written to every block.
+//
+// GB300 mapping: a block takes (genome, chunk of pairs), bulk-copies the
+// genome's record into shared memory once (TMA + mbarrier), and lists the
+// nodes that the output depends on, walking the levels back from it; only
+// these are evaluated and have a row in the value tile.  Each thread evaluates
+// 4 consecutive pairs at a time in its own four adjacent columns.  Node and
+// edge reads are the same for the whole warp (broadcasts), the four values of
+// a source are one 16-byte read, and the sums run as packed pairs
+// (fma.rn.f32x2: two IEEE fused multiply-adds per instruction, each rounded as
+// the scalar one, so the bits are those of every other path).  No barrier is
+// needed between nodes.  A block has as many threads at work as its tile has
+// room for: 256 up to 16 rows, 128 at 32.
+//
+// Bound by issue (66% of the slots at 22 warps per SM): the edges' shared
+// memory reads, the dispatches and the transcendentals; the only traffic is 4
+// bytes written per weight.  1000 genomes (up to 32 nodes, 96 connections), 3
+// layers of 16 x 16: 0.36 ms and 0.23 G warp instructions, 1.45 TB/s written.
+// One pair per thread and column, every node, every block evaluated: 2.70 ms
+// and 3.07 G; four columns and one evaluation per pair, without the list of
+// needed nodes and with a fixed 128 threads: 1.29 ms and 0.75 G at 12 warps.
+#include <algorithm>
+
 #include "neat_device.cuh"
 #include "neat_internal.h"
 #include "neat_trace.h"
@@ -24,147 +41,352 @@ namespace neat {
 namespace {
 
 constexpr int kCppnThreads = 256;
-constexpr int kCppnQueriesPerThread = 16;
+constexpr int kCppnMaxNodes = 256;   // above what shared memory admits (195)
 
 struct CppnArgs {
     const uint8_t *rec;
     size_t stride;
     float *out;
     int pop, N;
-    int res, layers;
-    long queries;            // per genome
-    int chunks;              // blocks per genome
+    int res, blocks;         // weight blocks (layers - 1)
+    int pairs;               // res^4: weights per block
+    int chunk, chunks;       // pairs per thread block, thread blocks per genome
     float threshold;
     int rec_words;           // 16-byte words of the record region
+    int edge_words;          // 16-byte words of the widened edges (0: edges stay as they are in the record)
+    int tile_bytes;          // value tile
     int use_xy;              // node coordinate table in shared memory (res^2 <= 4096)
+    int vec_out;             // weights written 16 bytes at a time
 };
 
 __device__ unsigned int g_cppn_error;
 
-// QPT: queries per thread evaluated together (1, or 2 in columns tid and
-// tid + 256 of a 512-column tile, sharing each node's entry, dispatch and
-// edge entries); every query's value is bit-equal either way.
-template <int QPT>
+// ---- pairs of floats in 64-bit registers (PTX f32x2 arithmetic)
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 pack2(float x, float y)
+{
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c)
+{
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b)
+{
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// An edge as staged: weight (twice, when widened) and the byte offset of its
+// source's row of the value tile.
+template <bool WIDE>
+struct Edge;
+template <>
+struct Edge<true> {
+    using T = uint4;
+    static __device__ __forceinline__ f2 ww(const uint4 &e) { return pack2(__uint_as_float(e.x), __uint_as_float(e.y)); }
+    static __device__ __forceinline__ float w(const uint4 &e) { return __uint_as_float(e.x); }
+    static __device__ __forceinline__ uint32_t at(const uint4 &e) { return e.z; }
+};
+template <>
+struct Edge<false> {
+    using T = uint2;
+    static __device__ __forceinline__ f2 ww(const uint2 &e) { return pack2(__uint_as_float(e.x), __uint_as_float(e.x)); }
+    static __device__ __forceinline__ float w(const uint2 &e) { return __uint_as_float(e.x); }
+    static __device__ __forceinline__ uint32_t at(const uint2 &e) { return e.y; }
+};
+
+// The thread's four values of the tile row at byte offset `at` (v: the
+// thread's columns).
+struct Four {
+    f2 lo, hi;
+};
+__device__ __forceinline__ Four load4(const char *v, uint32_t at)
+{
+    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(v + at);
+    return Four{x.x, x.y};
+}
+
+// Sums of a node's edges for the thread's four columns: edge i into partial
+// i mod 4 from +0 with fused multiply-adds, then (p0 + p1) + (p2 + p3), the
+// order of every evaluation path.
+template <bool WIDE, int EC>
+__device__ __forceinline__ Four sum_fixed(const typename Edge<WIDE>::T *__restrict__ e, const char *__restrict__ v)
+{
+    Four q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) q[k] = Four{0ull, 0ull};
+#pragma unroll
+    for (int i = 0; i < EC; ++i) {
+        const auto t = e[i];
+        const f2 w = Edge<WIDE>::ww(t);
+        const Four x = load4(v, Edge<WIDE>::at(t));
+        q[i & 3].lo = fma2(w, x.lo, q[i & 3].lo);
+        q[i & 3].hi = fma2(w, x.hi, q[i & 3].hi);
+    }
+    return Four{add2(add2(q[0].lo, q[1].lo), add2(q[2].lo, q[3].lo)),
+                add2(add2(q[0].hi, q[1].hi), add2(q[2].hi, q[3].hi))};
+}
+
+template <bool WIDE>
+__device__ __forceinline__ Four sum_any(const typename Edge<WIDE>::T *__restrict__ e, int ec, const char *__restrict__ v)
+{
+    Four q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) q[k] = Four{0ull, 0ull};
+    for (int i = 0; i < ec; i += 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k >= ec) break;                        // uniform over the block
+            const auto t = e[i + k];
+            const f2 w = Edge<WIDE>::ww(t);
+            const Four x = load4(v, Edge<WIDE>::at(t));
+            q[k].lo = fma2(w, x.lo, q[k].lo);
+            q[k].hi = fma2(w, x.hi, q[k].hi);
+        }
+    }
+    return Four{add2(add2(q[0].lo, q[1].lo), add2(q[2].lo, q[3].lo)),
+                add2(add2(q[0].hi, q[1].hi), add2(q[2].hi, q[3].hi))};
+}
+
+template <bool WIDE>
+__device__ __forceinline__ Four sum_edges(const typename Edge<WIDE>::T *__restrict__ e, int ec,
+                                          const char *__restrict__ v)
+{
+    switch (ec) {
+    case 0: return Four{0ull, 0ull};
+    case 1: return sum_fixed<WIDE, 1>(e, v);
+    case 2: return sum_fixed<WIDE, 2>(e, v);
+    case 3: return sum_fixed<WIDE, 3>(e, v);
+    case 4: return sum_fixed<WIDE, 4>(e, v);
+    case 5: return sum_fixed<WIDE, 5>(e, v);
+    case 6: return sum_fixed<WIDE, 6>(e, v);
+    case 7: return sum_fixed<WIDE, 7>(e, v);
+    case 8: return sum_fixed<WIDE, 8>(e, v);
+    default: return sum_any<WIDE>(e, ec, v);
+    }
+}
+
+// Products or maxima, the same partials.
+template <bool WIDE, uint32_t AGG>
+__device__ __forceinline__ void fold_edges(const typename Edge<WIDE>::T *__restrict__ e, int ec,
+                                           const char *__restrict__ v, float out[4])
+{
+    float q[4][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q[k][j] = agg_identity(AGG);
+    for (int i = 0; i < ec; i += 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k >= ec) break;
+            const auto t = e[i + k];
+            const float w = Edge<WIDE>::w(t);
+            const float4 x = *reinterpret_cast<const float4 *>(v + Edge<WIDE>::at(t));
+            q[k][0] = agg_step(AGG, q[k][0], w, x.x);
+            q[k][1] = agg_step(AGG, q[k][1], w, x.y);
+            q[k][2] = agg_step(AGG, q[k][2], w, x.z);
+            q[k][3] = agg_step(AGG, q[k][3], w, x.w);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        out[j] = agg_combine(AGG, agg_combine(AGG, q[0][j], q[1][j]), agg_combine(AGG, q[2][j], q[3][j]));
+}
+
+template <bool WIDE>
 __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
 {
     extern __shared__ __align__(16) uint4 smem[];
     __shared__ uint64_t bar_mem;
-    __shared__ float coord[NEAT_MAX_NODES];
-    const int tid = threadIdx.x;
+    __shared__ float coord[256];
+    __shared__ uint8_t need[kCppnMaxNodes], slot_of[kCppnMaxNodes];
+    __shared__ int failed, n_prog;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
     const int g = (int)(blockIdx.x / a.chunks);
-    const long q0 = (long)(blockIdx.x - (long)g * a.chunks) * (kCppnThreads * kCppnQueriesPerThread);
+    const int q0 = (int)(blockIdx.x - (unsigned)g * a.chunks) * a.chunk;
     uint4 *srec = smem;
-    float *v = reinterpret_cast<float *>(smem + a.rec_words);
-    float2 *nodexy = reinterpret_cast<float2 *>(v + (size_t)a.N * kCppnThreads * QPT);   // (x, y) of node i
+    uint4 *prog = srec + a.rec_words;                      // [N] the nodes to evaluate
+    uint4 *wide = prog + a.N;
+    char *tile = reinterpret_cast<char *>(wide + a.edge_words);
+    float2 *nodexy = reinterpret_cast<float2 *>(tile + a.tile_bytes);   // (x, y) of node i
     const uint32_t bar = smem_addr(&bar_mem);
     const uint8_t *grec = a.rec + (size_t)g * a.stride;
     if (tid == 0) {
         const uint32_t bytes = min(align16(__ldg(reinterpret_cast<const uint32_t *>(grec) + 4)),
                                    (uint32_t)a.rec_words * 16u);
+        failed = 0;
         mbar_init(bar, 1);
         mbar_arrive_expect_tx(bar, bytes);
         bulk_g2s(smem_addr(srec), grec, bytes, bar);
     }
-    for (int i = tid; i < a.res; i += kCppnThreads)
-        coord[i] = (float)(-1.0 + 2.0 * (double)i / (double)(a.res - 1));
+    for (int i = tid; i < a.res; i += nt) coord[i] = (float)(-1.0 + 2.0 * (double)i / (double)(a.res - 1));
+    for (int i = tid; i < kCppnMaxNodes; i += nt) need[i] = 0;
     __syncthreads();
+    const int rr = a.res * a.res;
     if (a.use_xy)
-        for (int i = tid; i < a.res * a.res; i += kCppnThreads) nodexy[i] = make_float2(coord[i % a.res], coord[i / a.res]);
-    __shared__ int failed;
-    if (tid == 0) failed = 0;
-    __syncthreads();
+        for (int i = tid; i < rr; i += nt) nodexy[i] = make_float2(coord[i % a.res], coord[i / a.res]);
     if (!mbar_wait(bar, 0)) failed = 1;
     __syncthreads();
-    float *out = a.out + (size_t)g * a.queries;
-    const long qend = min(a.queries, q0 + (long)kCppnThreads * kCppnQueriesPerThread);
-    if (failed) {
-        if (tid == 0) atomicOr(&g_cppn_error, kErrWaitExpired);
-        mbar_wait(bar, 0);
-        for (long q = q0 + tid; q < qend; q += kCppnThreads) out[q] = __int_as_float(0x7fc00000);
-        return;
-    }
+    float *out = a.out + (size_t)g * a.blocks * (size_t)a.pairs;
+    const int qend = min(a.pairs, q0 + a.chunk);
     const uint4 h0 = srec[0], h1 = srec[1];
-    if (h0.z & NEAT_G_ERROR_MASK) {
-        for (long q = q0 + tid; q < qend; q += kCppnThreads) out[q] = __int_as_float(0x7fc00000);
+    if (failed || (h0.z & NEAT_G_ERROR_MASK)) {
+        if (failed && tid == 0) atomicOr(&g_cppn_error, kErrWaitExpired);
+        if (failed) mbar_wait(bar, 0);                     // let the copy land before the block's memory is released
+        for (int l = 0; l < a.blocks; ++l)
+            for (int q = q0 + tid; q < qend; q += nt) out[(size_t)l * a.pairs + q] = __int_as_float(0x7fc00000);
         return;
     }
-    const int n_nodes = (int)(h0.x & 0xffffu);
-    const int first = (int)(h0.w >> 16);               // leading input positions need no evaluation
-    const bool sum_only = ((h0.w >> 8) & 0xffu) == 0u;  // uniform sum aggregation
+    const int n_nodes = (int)(h0.x & 0xffffu), n_levels = (int)(h0.x >> 16), n_edges = (int)h0.y;
     const uint4 *nodes = srec + 2;
-    const uint2 *edges = reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(srec) + h1.y);
+    uint2 *packed = reinterpret_cast<uint2 *>(reinterpret_cast<char *>(srec) + h1.y);
+    const uint16_t *lev = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.z);
     const uint16_t *io = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.w);
-    constexpr int lgT = QPT == 2 ? 9 : 8;               // value slot = (p << lgT) + column
-    static_assert((1 << lgT) == kCppnThreads * QPT, "tile of the CPPN value array");
-    const int pin0 = io[0], pin1 = io[1], pin2 = io[2], pin3 = io[3], pin4 = io[4], pout = io[5];
-    const int per_block = a.res * a.res * a.res * a.res;
-    const int rr = a.res * a.res;
-    // (source, target) of this thread's first query; later queries advance
-    // it by kCppnThreads without dividing
-    int r = (int)((q0 + tid) % per_block);
-    int s = r / rr, t = r - s * rr;
-    auto advance = [&](int &r_, int &s_, int &t_) {
-        r_ += kCppnThreads;
-        t_ += kCppnThreads;
-        if (r_ >= per_block) {                         // into the next layer block
-            r_ -= per_block;
-            s_ = r_ / rr;
-            t_ = r_ - s_ * rr;
-        } else {
-            while (t_ >= rr) {
-                t_ -= rr;
-                ++s_;
+    const int p_out = io[5];
+    if (tid < 32) {
+        // the nodes that the output depends on, from the last level back
+        if (lane == 0) need[p_out] = 1;
+        __syncwarp();
+        for (int l = n_levels - 1; l > 0; --l) {
+            for (int p = lev[l] + lane; p < lev[l + 1]; p += 32)
+                if (need[p]) {
+                    const uint32_t z = nodes[p].z;
+                    for (uint32_t i = z & 0xffffu, e = i + (z >> 16); i < e; ++i) need[packed[i].y] = 1;
+                }
+            __syncwarp();
+        }
+        // tile rows: the inputs, then the nodes to evaluate in their order
+        if (lane < 5) slot_of[io[lane]] = (uint8_t)lane;
+        int count = 0;
+        for (int p = lane; p - lane < n_nodes; p += 32) {
+            const uint4 ne = p < n_nodes ? nodes[p] : make_uint4(0u, 0u, 0u, (uint32_t)kInputAct);
+            const bool used = (ne.w & 0xffu) != kInputAct && need[p];
+            const unsigned m = __ballot_sync(0xffffffffu, used);
+            if (used) {
+                const int k = count + __popc(m & ((1u << lane) - 1u));
+                prog[k] = ne;
+                slot_of[p] = (uint8_t)(5 + k);
             }
+            count += __popc(m);
         }
-    };
-    auto put_inputs = [&](int s_, int t_, int col) {
-        float2 ps, pt;
-        if (a.use_xy) {
-            ps = nodexy[s_];
-            pt = nodexy[t_];
-        } else {
-            ps = make_float2(coord[s_ % a.res], coord[s_ / a.res]);
-            pt = make_float2(coord[t_ % a.res], coord[t_ / a.res]);
-        }
-        v[(pin0 << lgT) + col] = ps.x;
-        v[(pin1 << lgT) + col] = ps.y;
-        v[(pin2 << lgT) + col] = pt.x;
-        v[(pin3 << lgT) + col] = pt.y;
-        v[(pin4 << lgT) + col] = 1.0f;
-    };
-    for (long q = q0 + tid; q < qend; q += (long)kCppnThreads * QPT) {
-        put_inputs(s, t, tid);
-        if (QPT == 2) {
-            int r2 = r, s2 = s, t2 = t;
-            advance(r2, s2, t2);                       // the thread's next query, in column tid + 256
-            put_inputs(s2, t2, tid + kCppnThreads);
-            if (sum_only) {
-                for (int p = first; p < n_nodes; ++p)
-                    eval_node_sum_by_count2(nodes[p], edges, v, p, lgT, tid, kCppnThreads);
-            } else {
-                for (int p = first; p < n_nodes; ++p) {
-                    eval_node_tile<false>(nodes[p], edges, v, p, lgT, tid);
-                    eval_node_tile<false>(nodes[p], edges, v, p, lgT, tid + kCppnThreads);
+        if (lane == 0) n_prog = count;
+    }
+    __syncthreads();
+    // four columns per thread, as many threads as the rows leave room for
+    const int np = n_prog;
+    const int active = min(nt, (a.tile_bytes / (16 * (5 + np))) & ~31);
+    const int row = 16 * active;                           // bytes of a tile row
+    // sources become byte offsets of their rows (a node that is not evaluated
+    // has edges no one reads)
+    for (int i = tid; i < n_edges; i += nt) {
+        const uint2 e = packed[i];
+        const uint32_t at = (uint32_t)(slot_of[e.y] * row);
+        if (WIDE) wide[i] = make_uint4(e.x, e.x, at, 0u);
+        else packed[i].y = at;
+    }
+    __syncthreads();
+    if (tid >= active) return;
+    using E = typename Edge<WIDE>::T;
+    const E *edges = WIDE ? reinterpret_cast<const E *>(wide) : reinterpret_cast<const E *>(packed);
+    char *v = tile + 16 * tid;                             // the thread's columns
+    *reinterpret_cast<float4 *>(v + 4 * row) = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+    for (int q = q0 + 4 * tid; q < qend; q += 4 * active) {
+        {
+            int s = q / rr, t = q - s * rr;
+            float2 ps[4], pt[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (a.use_xy) {
+                    ps[j] = nodexy[s];
+                    pt[j] = nodexy[t];
+                } else {
+                    ps[j] = make_float2(coord[s % a.res], coord[s / a.res]);
+                    pt[j] = make_float2(coord[t % a.res], coord[t / a.res]);
+                }
+                if (++t == rr) {
+                    t = 0;
+                    if (s + 1 < rr) ++s;                   // past the last pair: any source will do
                 }
             }
-            const float w = v[(pout << lgT) + tid];
-            out[q] = (fabsf(w) < a.threshold) ? 0.0f : w;
-            if (q + kCppnThreads < qend) {
-                const float w2 = v[(pout << lgT) + tid + kCppnThreads];
-                out[q + kCppnThreads] = (fabsf(w2) < a.threshold) ? 0.0f : w2;
+            *reinterpret_cast<float4 *>(v) = make_float4(ps[0].x, ps[1].x, ps[2].x, ps[3].x);
+            *reinterpret_cast<float4 *>(v + row) = make_float4(ps[0].y, ps[1].y, ps[2].y, ps[3].y);
+            *reinterpret_cast<float4 *>(v + 2 * row) = make_float4(pt[0].x, pt[1].x, pt[2].x, pt[3].x);
+            *reinterpret_cast<float4 *>(v + 3 * row) = make_float4(pt[0].y, pt[1].y, pt[2].y, pt[3].y);
+        }
+        char *vp = v + 5 * row;
+        float4 y = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        uint4 next = prog[0];
+        for (int p = 0; p < np; ++p, vp += row) {
+            const uint4 ne = next;
+            next = prog[min(p + 1, np - 1)];               // read ahead of this node's sums
+            const uint32_t act = ne.w & 0xffu, agg = (ne.w >> 8) & 0xffu;
+            const int ec = (int)(ne.z >> 16);
+            const E *e = edges + (ne.z & 0xffffu);
+            f2 lo, hi;
+            if (agg == kAggSum) {
+                const Four sum = sum_edges<WIDE>(e, ec, v);
+                lo = sum.lo;
+                hi = sum.hi;
+            } else {
+                float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                if (ec > 0) {
+                    if (agg == kAggProduct) fold_edges<WIDE, kAggProduct>(e, ec, v, x);
+                    else if (agg == kAggMax) fold_edges<WIDE, kAggMax>(e, ec, v, x);
+                    else {
+                        const Four sum = sum_edges<WIDE>(e, ec, v);
+                        const float2 l2 = unpack2(sum.lo), h2 = unpack2(sum.hi);
+                        x[0] = l2.x / (float)ec;
+                        x[1] = l2.y / (float)ec;
+                        x[2] = h2.x / (float)ec;
+                        x[3] = h2.y / (float)ec;
+                    }
+                }
+                lo = pack2(x[0], x[1]);
+                hi = pack2(x[2], x[3]);
             }
-            r = r2;
-            s = s2;
-            t = t2;
-            advance(r, s, t);
-        } else {
-            if (sum_only)
-                for (int p = first; p < n_nodes; ++p) eval_node_sum_by_count<false>(nodes[p], edges, v, p, lgT, tid);
-            else
-                for (int p = first; p < n_nodes; ++p) eval_node_tile<false>(nodes[p], edges, v, p, lgT, tid);
-            const float w = v[(pout << lgT) + tid];
-            out[q] = (fabsf(w) < a.threshold) ? 0.0f : w;
-            advance(r, s, t);
+            const f2 rr2 = pack2(__uint_as_float(ne.y), __uint_as_float(ne.y));
+            const f2 bb2 = pack2(__uint_as_float(ne.x), __uint_as_float(ne.x));
+            const float2 z0 = unpack2(fma2(rr2, lo, bb2)), z1 = unpack2(fma2(rr2, hi, bb2));
+            switch (act) {                                 // one dispatch for the four columns
+            case 1: y = make_float4(activate(1, z0.x), activate(1, z0.y), activate(1, z1.x), activate(1, z1.y)); break;
+            case 2: y = make_float4(activate(2, z0.x), activate(2, z0.y), activate(2, z1.x), activate(2, z1.y)); break;
+            case 3: y = make_float4(activate(3, z0.x), activate(3, z0.y), activate(3, z1.x), activate(3, z1.y)); break;
+            case 4: y = make_float4(activate(4, z0.x), activate(4, z0.y), activate(4, z1.x), activate(4, z1.y)); break;
+            case 5: y = make_float4(activate(5, z0.x), activate(5, z0.y), activate(5, z1.x), activate(5, z1.y)); break;
+            case 6: y = make_float4(activate(6, z0.x), activate(6, z0.y), activate(6, z1.x), activate(6, z1.y)); break;
+            default: y = make_float4(z0.x, z0.y, z1.x, z1.y);
+            }
+            *reinterpret_cast<float4 *>(vp) = y;
+        }
+        // the output is the last node that anything needed is evaluated for
+        float4 w = y;
+        w.x = fabsf(w.x) < a.threshold ? 0.0f : w.x;
+        w.y = fabsf(w.y) < a.threshold ? 0.0f : w.y;
+        w.z = fabsf(w.z) < a.threshold ? 0.0f : w.z;
+        w.w = fabsf(w.w) < a.threshold ? 0.0f : w.w;
+        for (int l = 0; l < a.blocks; ++l) {
+            float *o = out + (size_t)l * a.pairs + q;
+            if (a.vec_out) {
+                *reinterpret_cast<float4 *>(o) = w;
+            } else {
+                o[0] = w.x;
+                if (q + 1 < qend) o[1] = w.y;
+                if (q + 2 < qend) o[2] = w.z;
+                if (q + 3 < qend) o[3] = w.w;
+            }
         }
     }
 }
@@ -196,25 +418,34 @@ extern "C" int neat_cppn_query(const void *transformed_dev, int32_t pop, neat_di
     a.pop = pop;
     a.N = d.max_nodes;
     a.res = sub.resolution;
-    a.layers = sub.layers;
+    a.blocks = sub.layers - 1;
     const long r2 = (long)sub.resolution * sub.resolution;
-    a.queries = (long)(sub.layers - 1) * r2 * r2;
-    const long per_block = (long)kCppnThreads * kCppnQueriesPerThread;
-    a.chunks = (int)((a.queries + per_block - 1) / per_block);
+    a.pairs = (int)(r2 * r2);                              // at most 181^4 < 2^31
+    // pairs per block: fewer prologues, but about eight blocks per resident
+    // one (three per SM) before blocks grow
+    a.chunk = 16384;
+    while (a.chunk > 1024 && (long)pop * ((a.pairs + a.chunk - 1) / a.chunk) < 8L * 3 * 152) a.chunk >>= 1;
+    a.chunks = (a.pairs + a.chunk - 1) / a.chunk;
     a.threshold = threshold;
     a.rec_words = (int)(record_max_bytes(5, 1, d.max_nodes, d.max_conns) / 16);
     a.use_xy = (r2 <= 4096) ? 1 : 0;
-    // two queries per thread where the doubled value tile fits, else one
-    auto smem_for = [&](int qpt) {
-        return (size_t)a.rec_words * 16 + 4u * (size_t)d.max_nodes * kCppnThreads * qpt +
-               (a.use_xy ? 8u * (size_t)r2 : 0u);
+    a.vec_out = (a.pairs % 4 == 0 && (reinterpret_cast<uintptr_t>(weights_dev) & 15u) == 0) ? 1 : 0;
+    // the value tile: 64 KB (three blocks per SM), or 128 columns of every
+    // node where that is more; edges widened where there is room
+    a.tile_bytes = std::max(64 * 1024, 512 * d.max_nodes);
+    const size_t limit = 200u * 1024u;
+    auto smem_for = [&](bool wide) {
+        return 16u * ((size_t)a.rec_words + (size_t)d.max_nodes + (wide ? (size_t)d.max_conns : 0u)) +
+               (size_t)a.tile_bytes + (a.use_xy ? 8u * (size_t)r2 : 0u);
     };
-    const int qpt = smem_for(2) <= 200u * 1024u ? 2 : 1;
-    const size_t smem = smem_for(qpt);
-    if (smem > 200u * 1024u) return invalid("neat_cppn_query: genome too large for one block (max_nodes <= 160)");
+    if ((size_t)a.rec_words * 16 + 1024u * (size_t)d.max_nodes + (a.use_xy ? 8u * (size_t)r2 : 0u) > limit)
+        return invalid("neat_cppn_query: genome too large for one block (max_nodes <= 160)");
+    const bool wide = smem_for(true) <= limit;
+    a.edge_words = wide ? d.max_conns : 0;
+    const size_t smem = smem_for(wide);
     const long blocks = (long)pop * a.chunks;
     if (blocks > 0x7fffffffL) return invalid("neat_cppn_query: too many queries");
-    auto kern = qpt == 2 ? cppn_kernel<2> : cppn_kernel<1>;
+    auto kern = wide ? cppn_kernel<true> : cppn_kernel<false>;
     int rc = allow_dynamic_smem(reinterpret_cast<const void *>(kern), smem, "neat_cppn_query: shared memory per block");
     if (rc) return rc;
     kern<<<(unsigned)blocks, kCppnThreads, smem, as_stream(stream)>>>(a);
