@@ -61,33 +61,6 @@ struct CppnArgs {
 
 __device__ unsigned int g_cppn_error;
 
-// ---- pairs of floats in 64-bit registers (PTX f32x2 arithmetic)
-using f2 = unsigned long long;
-__device__ __forceinline__ f2 pack2(float x, float y)
-{
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f2 v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c)
-{
-    f2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f2 add2(f2 a, f2 b)
-{
-    f2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
 // An edge as staged: weight (twice, when widened) and the byte offset of its
 // source's row of the value tile.
 template <bool WIDE>

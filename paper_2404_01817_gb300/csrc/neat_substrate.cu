@@ -20,6 +20,11 @@
 // the HBM roofline at one vector per genome); shapes it cannot take (R not a
 // multiple of 4) use per-thread VEC-wide read-only loads (substrate_kernel).
 // Both accumulate compensated dot products and give the same bits.
+//
+// Bounds: at one vector per genome the weights' stream (1000 genomes of 3
+// layers of 16 x 16: 90 us, 5.8 TB/s); at 16 the ten FP32 operations of a
+// compensated step, run as packed pairs so that they take half the issue
+// slots: 0.74 ms, 74% of the FP32 lanes (scalar 0.92 ms, 59%).
 #include <algorithm>
 
 #include "neat_device.cuh"
@@ -40,6 +45,7 @@ struct SubArgs {
     int groups;            // slices of the source range (threads per column group)
     int cols;              // column groups per pass (cols * groups <= threads)
     int stage_rows;        // bulk-copy path: source rows per shared-memory stage
+    int tiles;             // vector tiles per genome
 };
 
 __device__ unsigned int g_substrate_error;
@@ -66,6 +72,20 @@ __device__ __forceinline__ void dot2_step(float &s, float &c, float x, float w)
     two_sum(s, p, t, e);
     s = t;
     c = __fadd_rn(c, __fadd_rn(e, pe));
+}
+
+// dot2_step on two accumulators at once, x2 * w2 half by half, nw2 = -w2: the
+// operations of dot2_step with the product's error held negated (p - x*w
+// exactly), so c takes e - (-pe); the same bits in half the issue slots.
+__device__ __forceinline__ void dot2_step2(f2 &s, f2 &c, f2 x2, f2 w2, f2 nw2)
+{
+    const f2 p = mul2(x2, w2);
+    const f2 npe = fma2(x2, nw2, p);
+    const f2 t = add2(s, p);
+    const f2 z = sub2(t, s);
+    const f2 e = add2(sub2(s, sub2(t, z)), sub2(p, z));
+    s = t;
+    c = add2(c, sub2(e, npe));
 }
 
 // The slices' (s, c) pairs added in slice order, rounded once at the end.
@@ -106,7 +126,8 @@ __global__ void __launch_bounds__(kSubThreads) substrate_kernel(const SubArgs a)
     float *nxt = cur + NB * R;             // [NB][R]
     float *ps = nxt + NB * R;              // [groups][NB][R] slice sums
     float *pc = ps + (size_t)a.groups * NB * R;   // [groups][NB][R] their rounding errors
-    const int g = blockIdx.x, b0 = blockIdx.y * NB;
+    // a genome's vector tiles are neighbours in the grid: they share its weights in L2
+    const int g = blockIdx.x / a.tiles, b0 = (blockIdx.x - g * a.tiles) * NB;
     const int nb = min(NB, a.B - b0);
     const int tid = threadIdx.x;
     const float *xg = a.x + ((size_t)g * a.B + b0) * R;
@@ -122,30 +143,62 @@ __global__ void __launch_bounds__(kSubThreads) substrate_kernel(const SubArgs a)
         for (int c0 = 0; c0 < ncols; c0 += a.cols) {
             const int c = c0 + col_in_pass;
             if (grp < a.groups && c < ncols) {
-                float as[NB][VEC], ac[NB][VEC];
+                // accumulators in pairs: of columns, or of vectors where a thread
+                // has one column; a lone vector's single column stays scalar
+                constexpr bool kPairs = NB * VEC > 1;
+                constexpr int kAcc = kPairs ? NB * VEC / 2 : 1;
+                f2 as[kAcc], ac[kAcc];
+                float s1f = 0.0f, c1f = 0.0f;
 #pragma unroll
-                for (int b = 0; b < NB; ++b)
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) as[b][v] = ac[b][v] = 0.0f;
+                for (int k = 0; k < kAcc; ++k) as[k] = ac[k] = 0ull;
                 const int s0 = grp * slice, s1 = min(R, s0 + slice);
                 const V *col = reinterpret_cast<const V *>(Wl) + c;
 #pragma unroll 8
                 for (int s = s0; s < s1; ++s) {
                     const V wv = __ldg(col + (size_t)s * ncols);
+                    if constexpr (!kPairs) {
+                        dot2_step(s1f, c1f, cur[s], VecT<VEC>::get(wv, 0));
+                    } else if constexpr (VEC == 1) {
+                        const f2 w2 = pack2(VecT<VEC>::get(wv, 0), VecT<VEC>::get(wv, 0)), nw2 = neg2(w2);
 #pragma unroll
-                    for (int b = 0; b < NB; ++b) {
-                        const float xv = cur[b * R + s];
+                        for (int b = 0; b < NB; b += 2)
+                            dot2_step2(as[b / 2], ac[b / 2], pack2(cur[b * R + s], cur[(b + 1) * R + s]), w2, nw2);
+                    } else {
+                        f2 w2[VEC / 2], nw2[VEC / 2];
 #pragma unroll
-                        for (int v = 0; v < VEC; ++v) dot2_step(as[b][v], ac[b][v], xv, VecT<VEC>::get(wv, v));
+                        for (int v = 0; v < VEC; v += 2) {
+                            w2[v / 2] = pack2(VecT<VEC>::get(wv, v), VecT<VEC>::get(wv, v + 1));
+                            nw2[v / 2] = neg2(w2[v / 2]);
+                        }
+#pragma unroll
+                        for (int b = 0; b < NB; ++b) {
+                            const f2 x2 = pack2(cur[b * R + s], cur[b * R + s]);
+#pragma unroll
+                            for (int k = 0; k < VEC / 2; ++k)
+                                dot2_step2(as[b * (VEC / 2) + k], ac[b * (VEC / 2) + k], x2, w2[k], nw2[k]);
+                        }
                     }
                 }
+                auto put = [&](int b, int v, float sum, float err) {
+                    ps[((size_t)grp * NB + b) * R + c * VEC + v] = sum;
+                    pc[((size_t)grp * NB + b) * R + c * VEC + v] = err;
+                };
+                if constexpr (!kPairs) {
+                    put(0, 0, s1f, c1f);
+                } else {
 #pragma unroll
-                for (int b = 0; b < NB; ++b)
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) {
-                        ps[((size_t)grp * NB + b) * R + c * VEC + v] = as[b][v];
-                        pc[((size_t)grp * NB + b) * R + c * VEC + v] = ac[b][v];
+                    for (int k = 0; k < kAcc; ++k) {
+                        const float2 sk = unpack2(as[k]), ck = unpack2(ac[k]);
+                        if constexpr (VEC == 1) {
+                            put(2 * k, 0, sk.x, ck.x);
+                            put(2 * k + 1, 0, sk.y, ck.y);
+                        } else {
+                            const int b = k / (VEC / 2), v = 2 * (k % (VEC / 2));
+                            put(b, v, sk.x, ck.x);
+                            put(b, v + 1, sk.y, ck.y);
+                        }
                     }
+                }
             }
             __syncthreads();
             // sum the slices in order, apply the activation
@@ -185,11 +238,14 @@ __global__ void __launch_bounds__(kSubThreads) substrate_tma_kernel(const SubArg
     __shared__ int failed;
     const int R = a.R, rows = a.stage_rows;
     float *stage = sm;                                      // [2][rows][R]
-    float *cur = stage + 2 * (size_t)rows * R;              // [NB][R]
-    float *nxt = cur + NB * R;                              // [NB][R]
-    float *ps = nxt + NB * R;                               // [groups][NB][R] slice sums
-    float *pc = ps + (size_t)(kSubThreads / (R / 4)) * NB * R;   // [groups][NB][R] their rounding errors
-    const int g = blockIdx.x, b0 = blockIdx.y * NB;
+    // values, each twice (both halves of a pair)
+    float2 *cur = reinterpret_cast<float2 *>(stage + 2 * (size_t)rows * R);   // [NB][R]
+    float2 *nxt = cur + NB * R;                                               // [NB][R]
+    // slice sums and their rounding errors [groups][NB][R], in the stages'
+    // memory once a layer's stages are used up
+    float *ps = stage, *pc = ps + (size_t)(kSubThreads / (R / 4)) * NB * R;
+    // a genome's vector tiles are neighbours in the grid: they share its weights in L2
+    const int g = blockIdx.x / a.tiles, b0 = (blockIdx.x - g * a.tiles) * NB;
     const int nb = min(NB, a.B - b0);
     const int tid = threadIdx.x;
     const int ncols = R / 4, groups = kSubThreads / ncols;
@@ -206,7 +262,10 @@ __global__ void __launch_bounds__(kSubThreads) substrate_tma_kernel(const SubArg
         failed = 0;
     }
     const float *xg = a.x + ((size_t)g * a.B + b0) * R;
-    for (int i = tid; i < NB * R; i += kSubThreads) cur[i] = (i < nb * R) ? __ldg(xg + i) : 0.0f;
+    for (int i = tid; i < NB * R; i += kSubThreads) {
+        const float v = (i < nb * R) ? __ldg(xg + i) : 0.0f;
+        cur[i] = make_float2(v, v);
+    }
     __syncthreads();
     // copies issued into and completions seen on each buffer (every thread
     // counts; thread 0 issues)
@@ -228,11 +287,9 @@ __global__ void __launch_bounds__(kSubThreads) substrate_tma_kernel(const SubArg
         const float *Wl = a.w + ((size_t)g * (a.L - 1) + l) * (size_t)R * R;
         const int act = (l + 2 == a.L) ? a.output_act : a.hidden_act;
         for (int st = 0; st < 2 && st < nstages; ++st) issue(st, Wl, st);
-        float as[NB][4], ac[NB][4];
+        f2 as[NB][2], ac[NB][2];
 #pragma unroll
-        for (int b = 0; b < NB; ++b)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) as[b][v] = ac[b][v] = 0.0f;
+        for (int b = 0; b < NB; ++b) as[b][0] = as[b][1] = ac[b][0] = ac[b][1] = 0ull;
         for (int st = 0; st < nstages; ++st) {
             const int buf = st & 1;
             if (mbar_wait(buf ? bar1 : bar0, (buf ? seen1 : seen0) & 1u)) {
@@ -241,18 +298,18 @@ __global__ void __launch_bounds__(kSubThreads) substrate_tma_kernel(const SubArg
                 failed = 1;
             }
             // this thread's rows: sources grp*slen + st*rps .. + rps - 1
-            const float4 *W4 = reinterpret_cast<const float4 *>(stage + (size_t)buf * rows * R +
-                                                                (size_t)grp * rps * R);
-            const float *xs = cur + grp * slen + st * rps;
+            const ulonglong2 *W4 = reinterpret_cast<const ulonglong2 *>(stage + (size_t)buf * rows * R +
+                                                                        (size_t)grp * rps * R) + col;
+            const f2 *xs = reinterpret_cast<const f2 *>(cur) + grp * slen + st * rps;
+#pragma unroll 2
             for (int r = 0; r < rps; ++r) {
-                const float4 w = W4[(size_t)r * ncols + col];
+                const ulonglong2 w = W4[(size_t)r * ncols];
+                const f2 nx = neg2(w.x), ny = neg2(w.y);
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
-                    const float xv = xs[b * R + r];
-                    dot2_step(as[b][0], ac[b][0], xv, w.x);
-                    dot2_step(as[b][1], ac[b][1], xv, w.y);
-                    dot2_step(as[b][2], ac[b][2], xv, w.z);
-                    dot2_step(as[b][3], ac[b][3], xv, w.w);
+                    const f2 x2 = xs[b * R + r];
+                    dot2_step2(as[b][0], ac[b][0], x2, w.x, nx);
+                    dot2_step2(as[b][1], ac[b][1], x2, w.y, ny);
                 }
             }
             __syncthreads();                                // every thread is done with the buffer
@@ -261,20 +318,18 @@ __global__ void __launch_bounds__(kSubThreads) substrate_tma_kernel(const SubArg
         }
         if (failed) break;
 #pragma unroll
-        for (int b = 0; b < NB; ++b)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                ps[((size_t)grp * NB + b) * R + col * 4 + v] = as[b][v];
-                pc[((size_t)grp * NB + b) * R + col * 4 + v] = ac[b][v];
-            }
-        __syncthreads();
-        for (int i = tid; i < NB * R; i += kSubThreads) {
-            const int b = i / R, t = i - b * R;
-            nxt[i] = activate((uint32_t)act, combine_slices(ps + (size_t)b * R + t, pc + (size_t)b * R + t,
-                                                             (size_t)NB * R, groups));
+        for (int b = 0; b < NB; ++b) {
+            const size_t at = ((size_t)grp * NB + b) * R + col * 4;
+            *reinterpret_cast<ulonglong2 *>(ps + at) = make_ulonglong2(as[b][0], as[b][1]);
+            *reinterpret_cast<ulonglong2 *>(pc + at) = make_ulonglong2(ac[b][0], ac[b][1]);
         }
         __syncthreads();
-        float *tmp = cur;
+        for (int i = tid; i < NB * R; i += kSubThreads) {
+            const float v = activate((uint32_t)act, combine_slices(ps + i, pc + i, (size_t)NB * R, groups));
+            nxt[i] = make_float2(v, v);
+        }
+        __syncthreads();
+        float2 *tmp = cur;
         cur = nxt;
         nxt = tmp;
     }
@@ -288,33 +343,44 @@ __global__ void __launch_bounds__(kSubThreads) substrate_tma_kernel(const SubArg
         for (int i = tid; i < nb * R; i += kSubThreads) yg[i] = __int_as_float(0x7fc00000);
         return;
     }
-    for (int i = tid; i < nb * R; i += kSubThreads) yg[i] = cur[i];
+    for (int i = tid; i < nb * R; i += kSubThreads) yg[i] = cur[i].x;
 }
 
 template <int NB, int VEC>
-int launch_sub(const SubArgs &a, int pop, cudaStream_t s)
+int launch_sub(SubArgs a, int pop, cudaStream_t s)
 {
     const size_t smem = sizeof(float) * ((size_t)2 * NB * a.R + 2 * (size_t)a.groups * NB * a.R);
     auto kern = substrate_kernel<NB, VEC>;
     int rc = allow_dynamic_smem(reinterpret_cast<const void *>(kern), smem, "neat_substrate_forward: shared memory");
     if (rc) return rc;
-    const dim3 grid((unsigned)pop, (unsigned)((a.B + NB - 1) / NB));
-    kern<<<grid, kSubThreads, smem, s>>>(a);
+    a.tiles = (a.B + NB - 1) / NB;
+    const long blocks = (long)pop * a.tiles;
+    if (blocks > 0x7fffffffL) return invalid("neat_substrate_forward: too many blocks");
+    kern<<<(unsigned)blocks, kSubThreads, smem, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "neat_substrate_forward: launch");
     return NEAT_OK;
 }
 
-template <int NB>
-int launch_tma(const SubArgs &a, int pop, cudaStream_t s)
+// Shared memory of the bulk-copy kernel: two stages (or the slice sums, which
+// take their place), two value tiles of pairs.
+size_t tma_smem_bytes(int R, int stage_rows, int nb)
 {
-    const size_t smem = sizeof(float) * (2 * (size_t)a.stage_rows * a.R + 2 * (size_t)NB * a.R +
-                                         2 * (size_t)(kSubThreads / (a.R / 4)) * NB * a.R);
+    const size_t stages = 2 * (size_t)stage_rows * R, sums = 2 * (size_t)(kSubThreads / (R / 4)) * nb * R;
+    return sizeof(float) * (std::max(stages, sums) + 4 * (size_t)nb * R);
+}
+
+template <int NB>
+int launch_tma(SubArgs a, int pop, cudaStream_t s)
+{
+    const size_t smem = tma_smem_bytes(a.R, a.stage_rows, NB);
     auto kern = substrate_tma_kernel<NB>;
     int rc = allow_dynamic_smem(reinterpret_cast<const void *>(kern), smem, "neat_substrate_forward: shared memory");
     if (rc) return rc;
-    const dim3 grid((unsigned)pop, (unsigned)((a.B + NB - 1) / NB));
-    kern<<<grid, kSubThreads, smem, s>>>(a);
+    a.tiles = (a.B + NB - 1) / NB;
+    const long blocks = (long)pop * a.tiles;
+    if (blocks > 0x7fffffffL) return invalid("neat_substrate_forward: too many blocks");
+    kern<<<(unsigned)blocks, kSubThreads, smem, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "neat_substrate_forward: launch");
     return NEAT_OK;
@@ -376,23 +442,22 @@ extern "C" int neat_substrate_forward(const float *weights_dev, int32_t pop, nea
     // bulk-copy path: 32 KB stages of whole source rows, tiles of up to 4
     // vectors (with the compensated sums, larger batches are bound by
     // arithmetic, not by streaming the weights once per tile), when R / 4
-    // divides the block and the stages, values and partial sums fit 112 KB
-    // (two or more blocks per SM).  Both kernels split the sources into the
-    // same slices, so their results are identical
+    // divides the block and a block takes at most 112 KB (two or more per SM;
+    // 16 KB stages and a third block at 4 vectors measured the same).  Both
+    // kernels split the sources into the same slices, so their
+    // results are identical
     if (vec4 && kSubThreads % (a.R / 4) == 0) {
         const int groups = kSubThreads / (a.R / 4);
-        // stage rows: about 32 KB, a multiple of the slices, each slice's
-        // share dividing the slice
+        const int nbt = std::min(nb, 4);
+        // stage rows: a multiple of the slices, each slice's share dividing
+        // the slice
         const int slen = a.R / groups;
         int rows = std::max(groups, std::min(a.R, (32 * 1024) / (4 * a.R)));
         while (rows > groups && (rows % groups || slen % (rows / groups))) --rows;
-        const int nbt = std::min(nb, 4);
-        const size_t smem = sizeof(float) * (2 * (size_t)rows * a.R + 2 * (size_t)nbt * a.R +
-                                             2 * (size_t)groups * nbt * a.R);
         // the same slices as substrate_kernel: groups = kSubThreads / (R / 4)
         // there too while its shared memory needs no fewer (true for nb <= 4)
         if (a.R % groups == 0 && rows % groups == 0 && slen % (rows / groups) == 0 && groups == a.groups &&
-            smem <= 112u * 1024u) {
+            tma_smem_bytes(a.R, rows, nbt) <= 112u * 1024u) {
             a.stage_rows = rows;
             switch (nbt) {
             case 1: return launch_tma<1>(a, pop, as_stream(stream));
