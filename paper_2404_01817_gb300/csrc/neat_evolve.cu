@@ -7,15 +7,23 @@
 // (u < T(p), T(p) = min(floor(p 2^32), 2^32)) and choose (floor(u k / 2^32)),
 // float normals give the perturbations.
 //
-// GB300 mapping: one block per genome, working in place on the population
-// tensors.  The node keys and the connections' (in, out, enabled) columns
-// are kept in shared memory while the four structural steps run one after
-// another (block-wide counts, rank selection by a block scan, first-free-row
-// searches, and for feedforward networks a key -> row hash table and a
-// breadth-first reachability sweep over the connections); the attribute step then updates every present row
-// in parallel.  Crossover: one block per child, the second parent's node
-// keys and (in, out) pairs in shared-memory hash tables (lowest row per key
-// or pair) looked up for every row of the first parent.
+// GB300 mapping: one warp per genome up to 128 node rows and 512 connection
+// rows (mutate_warp_kernel, crossover_warp_kernel), one block per genome
+// beyond.  The block forms work in place on the population tensors: the node
+// keys and the connections' (in, out, enabled) columns are kept in shared
+// memory while the four structural steps run one after another (block-wide
+// counts, rank selection by a block scan, first-free-row searches, and for
+// feedforward networks a key -> row hash table and a breadth-first
+// reachability sweep over the connections); the attribute step then updates
+// every present row in parallel.  Crossover: the second parent's node keys and
+// (in, out) pairs in shared-memory hash tables (lowest row per key or pair)
+// looked up for every row of the first parent.
+//
+// The warp forms are bound by memory latency (long-scoreboard stalls at 40 to
+// 45% of the warps, 34 to 45% of the issue slots).  10 000 Ant-sized genomes:
+// mutation 44 us (block of 64 threads per genome: 80 us, 3490 against 1510
+// warp instructions per genome), crossover 38 us (block of 128: 75 us, 4900
+// against 1710).
 #include <algorithm>
 
 #include "neat_device.cuh"
@@ -36,7 +44,7 @@ struct MutArgs {
     const uint32_t *words;
     const float *normals;
     const int32_t *new_keys;
-    int N, C, I, O, Np2;
+    int pop, N, C, I, O, Np2;
     size_t W, Z;                               // words / normals per genome
     unsigned long long t_node_add, t_node_delete, t_conn_add, t_conn_delete;
     unsigned long long t_bias_m, t_bias_mr, t_resp_m, t_resp_mr, t_w_m, t_w_mr, t_act, t_agg, t_en;
@@ -123,6 +131,272 @@ __device__ int select_choose(int R, Pred pred, uint32_t u, int *s_cnt, int *s_ro
         s_row, total_out, nullptr);
 }
 
+// ------------------------------------------------ a warp per genome
+//
+// Genomes of at most 128 node rows and 512 connection rows (predecessor masks
+// of four words, at most 14 KB a genome): one warp stages the whole genome in shared memory, so that the structural steps need warp
+// barriers only and the tensors are read and written once, in full sectors.
+// Candidate sets are bit masks (lane k holds rows 32k .. 32k+31), the cycle
+// check a sweep over predecessor masks.
+constexpr int kWarpNodes = 128, kWarpConns = 512;
+constexpr unsigned kAll = 0xffffffffu;
+
+// The mask of rows 32k .. 32k+31 of [0, R) that satisfy pred, on lane k.
+template <typename Pred>
+__device__ __forceinline__ uint32_t row_mask(int R, Pred pred, int lane)
+{
+    uint32_t mine = 0;
+    for (int k = 0; k * 32 < R; ++k) {
+        const int r = k * 32 + lane;
+        const unsigned m = __ballot_sync(kAll, r < R && pred(r));
+        if (lane == k) mine = m;
+    }
+    return mine;
+}
+
+__device__ __forceinline__ int mask_count(uint32_t mine) { return __reduce_add_sync(kAll, __popc(mine)); }
+
+// The row of rank `rank` (0 <= rank < count) in such a mask.
+__device__ __forceinline__ int mask_pick(uint32_t mine, int rank, int lane)
+{
+    int incl = __popc(mine);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kAll, incl, o);
+        if (lane >= o) incl += v;
+    }
+    const int owner = __ffs(__ballot_sync(kAll, rank < incl)) - 1;
+    int row = 0;
+    if (lane == owner) {
+        uint32_t m = mine;
+        for (int k = rank - (incl - __popc(mine)); k > 0; --k) m &= m - 1u;
+        row = lane * 32 + __ffs(m) - 1;
+    }
+    return __shfl_sync(kAll, row, owner);
+}
+
+// The lowest row of such a mask (-1 if none).
+__device__ __forceinline__ int mask_first(uint32_t mine)
+{
+    const unsigned some = __ballot_sync(kAll, mine != 0u);
+    if (some == 0u) return -1;
+    const int owner = __ffs(some) - 1;
+    return owner * 32 + __shfl_sync(kAll, __ffs(mine) - 1, owner);
+}
+
+struct MutWarpLayout {
+    int nodes, preds, ktab, total;           // byte offsets in a warp's shared memory (connections at 0)
+};
+__host__ __device__ inline MutWarpLayout mut_warp_layout(int N, int C, int Np2)
+{
+    MutWarpLayout l;
+    const int RN = (N + 31) / 32;
+    l.nodes = 16 * C;
+    l.preds = l.nodes + 20 * N;
+    l.ktab = l.preds + 4 * RN * N;
+    l.total = (l.ktab + 8 * Np2 + 15) & ~15;
+    return l;
+}
+
+__global__ void __launch_bounds__(128) mutate_warp_kernel(const MutArgs a)
+{
+    extern __shared__ __align__(16) unsigned char sm[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = blockIdx.x * (blockDim.x >> 5) + warp;
+    if (g >= a.pop) return;
+    const int N = a.N, C = a.C;
+    const MutWarpLayout lay = mut_warp_layout(N, C, a.Np2);
+    unsigned char *mine = sm + (size_t)warp * lay.total;
+    float4 *cs = reinterpret_cast<float4 *>(mine);                // [C] (in, out, enabled, weight)
+    float *ns = reinterpret_cast<float *>(mine + lay.nodes);      // [N][5]
+    float *nodes = a.nodes + (size_t)g * N * 5;
+    float4 *conns = reinterpret_cast<float4 *>(a.conns + (size_t)g * C * 4);
+    const uint32_t *u = a.words + (size_t)g * a.W;
+    const float *z = a.normals + (size_t)g * a.Z;
+
+    const uint32_t word = lane < 9 ? __ldg(u + lane) : 0u;        // the structural words
+#pragma unroll 4
+    for (int c = lane; c < C; c += 32) cs[c] = conns[c];
+#pragma unroll 4
+    for (int i = lane; i < 5 * N; i += 32) ns[i] = nodes[i];
+    __syncwarp();
+    auto u_at = [&](int k) { return __shfl_sync(kAll, word, k); };
+    auto node_present = [&](int r) { return !isnan(ns[5 * r]); };
+    auto conn_present = [&](int c) { return !(isnan(cs[c].x) || isnan(cs[c].y) || isnan(cs[c].z)); };
+    const float4 none = make_float4(qnan(), qnan(), qnan(), qnan());
+
+    // 1. node addition: split a present enabled connection
+    if (below(u_at(0), a.t_node_add)) {
+        const float nkey = (float)__ldg(a.new_keys + g);
+        const uint32_t enabled = row_mask(C, [&](int c) { return conn_present(c) && cs[c].z != 0.0f; }, lane);
+        uint32_t free = row_mask(C, [&](int c) { return !conn_present(c); }, lane);
+        const int total = mask_count(enabled);
+        const int rn = mask_first(row_mask(N, [&](int r) { return !node_present(r); }, lane));
+        const int ra = mask_first(free);
+        if (ra >= 0 && lane == (ra >> 5)) free &= free - 1u;
+        const int rb = mask_first(free);
+        bool used = false;
+        for (int r = lane; r < N; r += 32) used |= node_present(r) && ns[5 * r] == nkey;
+        used = __any_sync(kAll, used);
+        if (total > 0 && rn >= 0 && ra >= 0 && rb >= 0 && !used) {
+            const int pick = mask_pick(enabled, choose(u_at(1), total), lane);
+            __syncwarp();
+            if (lane == 0) {
+                const float4 old = cs[pick];
+                cs[pick].z = 0.0f;
+                cs[ra] = make_float4(old.x, nkey, 1.0f, 1.0f);
+                cs[rb] = make_float4(nkey, old.y, 1.0f, old.w);
+                float *n = ns + 5 * rn;
+                n[0] = nkey;
+                n[1] = a.bias_mean;
+                n[2] = a.resp_mean;
+                n[3] = (float)a.agg_default;
+                n[4] = (float)a.act_default;
+            }
+        }
+        __syncwarp();
+    }
+
+    // 2. node deletion: a hidden node and every connection touching it
+    if (below(u_at(2), a.t_node_delete)) {
+        const float io_end = (float)(a.I + a.O);
+        const uint32_t hidden = row_mask(N, [&](int r) { return node_present(r) && ns[5 * r] >= io_end; }, lane);
+        const int total = mask_count(hidden);
+        if (total > 0) {
+            const int rd = mask_pick(hidden, choose(u_at(3), total), lane);
+            const float q = ns[5 * rd];
+            for (int c = lane; c < C; c += 32)
+                if (conn_present(c) && (cs[c].x == q || cs[c].y == q)) cs[c] = none;
+            __syncwarp();
+            if (lane < 5) ns[5 * rd + lane] = qnan();
+            __syncwarp();
+        }
+    }
+
+    // 3. connection addition
+    if (below(u_at(4), a.t_conn_add)) {
+        const float in_end = (float)a.I;
+        const uint32_t here = row_mask(N, node_present, lane);
+        const uint32_t target = row_mask(N, [&](int r) { return node_present(r) && ns[5 * r] >= in_end; }, lane);
+        const int n_src = mask_count(here), n_dst = mask_count(target);
+        if (n_src > 0 && n_dst > 0) {
+            const float s = ns[5 * mask_pick(here, choose(u_at(5), n_src), lane)];
+            const float t = ns[5 * mask_pick(target, choose(u_at(6), n_dst), lane)];
+            const int existing = mask_first(
+                row_mask(C, [&](int c) { return conn_present(c) && cs[c].x == s && cs[c].y == t; }, lane));
+            __syncwarp();
+            if (existing >= 0) {
+                if (lane == 0) cs[existing].z = 1.0f;
+                __syncwarp();
+            } else {
+                bool reject = false;
+                if (a.feedforward && s == t) reject = true;
+                else if (a.feedforward) {
+                    // rows by key, then every row's predecessors among the
+                    // present nodes, then a sweep from t
+                    const int RN = (N + 31) >> 5;
+                    uint32_t *ktab = reinterpret_cast<uint32_t *>(mine + lay.ktab);    // [2 Np2]
+                    uint32_t *preds = reinterpret_cast<uint32_t *>(mine + lay.preds);  // [RN][N]
+                    const uint32_t kmask = 2u * (uint32_t)a.Np2 - 1u;
+                    const int kshift = __clz(kmask);
+                    for (int i = lane; i < 2 * a.Np2; i += 32) ktab[i] = kFree32;
+                    for (int i = lane; i < RN * N; i += 32) preds[i] = 0u;
+                    __syncwarp();
+                    for (int r = lane; r < N; r += 32)
+                        if (node_present(r)) insert32(ktab, kmask, kshift, (uint32_t)ns[5 * r] & 0xffffffu, (uint32_t)r);
+                    __syncwarp();
+                    auto row_of = [&](float k) { return find32(ktab, kmask, kshift, (uint32_t)k & 0xffffffu); };
+                    for (int c = lane; c < C; c += 32) {
+                        if (!conn_present(c)) continue;
+                        const int x = row_of(cs[c].x), y = row_of(cs[c].y);
+                        if (x >= 0 && y >= 0) atomicOr(preds + (x >> 5) * N + y, 1u << (x & 31));
+                    }
+                    __syncwarp();
+                    const int row_s = row_of(s), row_t = row_of(t);
+                    uint32_t seen = lane == (row_t >> 5) ? 1u << (row_t & 31) : 0u;    // lane k: rows 32k ..
+                    for (;;) {
+                        uint32_t next = seen;
+                        for (int k = 0; k < RN; ++k) {
+                            const int r = 32 * k + lane;
+                            uint32_t hit = 0;
+                            for (int j = 0; j < RN; ++j) {
+                                const uint32_t from = __shfl_sync(kAll, seen, j);
+                                if (r < N) hit |= preds[j * N + r] & from;
+                            }
+                            const unsigned m = __ballot_sync(kAll, hit != 0u);
+                            if (lane == k) next |= m;
+                        }
+                        const bool grown = __any_sync(kAll, next != seen);
+                        seen = next;
+                        reject = (__shfl_sync(kAll, seen, row_s >> 5) >> (row_s & 31)) & 1u;
+                        if (reject || !grown) break;
+                    }
+                }
+                if (!reject) {
+                    const int rf = mask_first(row_mask(C, [&](int c) { return !conn_present(c); }, lane));
+                    __syncwarp();
+                    if (rf >= 0 && lane == 0) cs[rf] = make_float4(s, t, 1.0f, fmaf(a.w_std, __ldg(z), a.w_mean));
+                    __syncwarp();
+                }
+            }
+        }
+    }
+
+    // 4. connection deletion
+    if (below(u_at(7), a.t_conn_delete)) {
+        const uint32_t present = row_mask(C, conn_present, lane);
+        const int total = mask_count(present);
+        if (total > 0) {
+            const int rc = mask_pick(present, choose(u_at(8), total), lane);
+            __syncwarp();
+            if (lane == 0) cs[rc] = none;
+            __syncwarp();
+        }
+    }
+
+    // attributes of every present row
+    const float in_end = (float)a.I;
+    const uint32_t *wc = u + kStructWords + 6 * (size_t)N;
+    const float *zc = z + kStructNormals + 2 * (size_t)N;
+#pragma unroll 4
+    for (int c = lane; c < C; c += 32) {
+        float4 x = cs[c];
+        const uint32_t w0 = __ldg(wc + 2 * (size_t)c);
+        const uint32_t w1 = a.t_en ? __ldg(wc + 2 * (size_t)c + 1) : 0xffffffffu;
+        const float zz = __ldg(zc + c);
+        if (!(isnan(x.x) || isnan(x.y) || isnan(x.z))) {
+            if (below(w0, a.t_w_m)) x.w = fmaf(a.w_power, zz, x.w);
+            else if (below(w0, a.t_w_mr)) x.w = fmaf(a.w_std, zz, a.w_mean);
+            if (a.t_en && below(w1, a.t_en)) x.z = (x.z != 0.0f) ? 0.0f : 1.0f;
+        }
+        conns[c] = x;
+    }
+    for (int r = lane; r < N; r += 32) {
+        float *n = ns + 5 * r;
+        if (isnan(n[0]) || n[0] < in_end) continue;
+        const uint32_t *w = u + kStructWords + 6 * (size_t)r;
+        const float *zz = z + kStructNormals + 2 * (size_t)r;
+        if (a.t_bias_m | a.t_bias_mr) {
+            const uint32_t w0 = __ldg(w);
+            const float z0 = __ldg(zz);
+            if (below(w0, a.t_bias_m)) n[1] = fmaf(a.bias_power, z0, n[1]);
+            else if (below(w0, a.t_bias_mr)) n[1] = fmaf(a.bias_std, z0, a.bias_mean);
+        }
+        if (a.t_resp_m | a.t_resp_mr) {
+            const uint32_t w1 = __ldg(w + 1);
+            const float z1 = __ldg(zz + 1);
+            if (below(w1, a.t_resp_m)) n[2] = fmaf(a.resp_power, z1, n[2]);
+            else if (below(w1, a.t_resp_mr)) n[2] = fmaf(a.resp_std, z1, a.resp_mean);
+        }
+        if (a.t_act && a.n_act > 0 && below(__ldg(w + 2), a.t_act)) n[4] = (float)a.act_opt[choose(__ldg(w + 3), a.n_act)];
+        if (a.t_agg && a.n_agg > 0 && below(__ldg(w + 4), a.t_agg)) n[3] = (float)a.agg_opt[choose(__ldg(w + 5), a.n_agg)];
+    }
+    __syncwarp();
+#pragma unroll 4
+    for (int i = lane; i < 5 * N; i += 32) nodes[i] = ns[i];
+}
+
+// ------------------------------------------------ larger: a block per genome
 __global__ void __launch_bounds__(kEvoThreads) mutate_kernel(const MutArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -343,6 +617,149 @@ __device__ __forceinline__ void write_empty_child(float *no, float4 *co, int N, 
     for (int c = lane; c < C; c += step) co[c] = make_float4(q, q, q, q);
 }
 
+// One warp per child, for parents of at most 128 node rows and 512 connection
+// rows.  The second parent's connections sit in a 32-bit table (22 bits of the
+// pair's hash | row); a lookup that matches reads the row it names, whose keys
+// decide and whose attributes are what the child takes.
+struct CrossWarpLayout {
+    int ntab, ctab, total;                   // byte offsets in a warp's shared memory (child's nodes at 0)
+};
+__host__ __device__ inline CrossWarpLayout cross_warp_layout(int N, int Np2, int Cp2)
+{
+    CrossWarpLayout l;
+    l.ntab = (20 * N + 15) & ~15;
+    l.ctab = l.ntab + 8 * Np2;               // 2 Np2 words
+    l.total = (l.ctab + 8 * Cp2 + 15) & ~15; // 2 Cp2 words
+    return l;
+}
+
+__device__ __forceinline__ uint32_t pair_hash(uint32_t ki, uint32_t ko)
+{
+    uint32_t h = ki * 0x9E3779B1u + ko * 0x85EBCA6Bu;
+    h ^= h >> 15;
+    h *= 0x2C1B3C6Du;
+    return h ^ (h >> 13);
+}
+
+__global__ void __launch_bounds__(128) crossover_warp_kernel(const CrossArgs a)
+{
+    extern __shared__ __align__(16) unsigned char sm[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int k = blockIdx.x * (blockDim.x >> 5) + warp;
+    if (k >= a.K) return;
+    const int N = a.N, C = a.C;
+    const CrossWarpLayout lay = cross_warp_layout(N, a.Np2, a.Cp2);
+    unsigned char *mine = sm + (size_t)warp * lay.total;
+    float *ns = reinterpret_cast<float *>(mine);                             // [N][5]
+    uint32_t *ntab = reinterpret_cast<uint32_t *>(mine + lay.ntab);          // key << 8 | lowest row of p2
+    uint32_t *ctab = reinterpret_cast<uint32_t *>(mine + lay.ctab);          // hash bits << 10 | lowest row of p2
+    const uint32_t nmask = 2u * (uint32_t)a.Np2 - 1u, cmask = 2u * (uint32_t)a.Cp2 - 1u;
+    const int nshift = __clz(nmask), cshift = __clz(cmask);
+    float *no = a.nodes_out + (size_t)k * N * 5;
+    float4 *co = reinterpret_cast<float4 *>(a.conns_out + (size_t)k * C * 4);
+    const int p1 = __ldg(a.parents + 2 * k), p2 = __ldg(a.parents + 2 * k + 1);
+    if (p1 < 0 || p1 >= a.pop || p2 < 0 || p2 >= a.pop) {
+        write_empty_child(no, co, N, C, lane, 32);
+        return;
+    }
+    const float *n1 = a.nodes + (size_t)p1 * N * 5, *n2 = a.nodes + (size_t)p2 * N * 5;
+    const float4 *c1 = reinterpret_cast<const float4 *>(a.conns + (size_t)p1 * C * 4);
+    const float4 *c2 = reinterpret_cast<const float4 *>(a.conns + (size_t)p2 * C * 4);
+    const uint32_t *w = a.words + (size_t)k * (N + C);
+    constexpr int kAhead = 4;                                                // rows loaded ahead per lane
+    float4 row[kAhead];
+    auto load_rows = [&](const float4 *from, int base) {
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            const int c = base + 32 * j + lane;
+            row[j] = make_float4(qnan(), 0.0f, 0.0f, 0.0f);
+            if (c < C) row[j] = __ldg(from + c);
+        }
+    };
+    load_rows(c2, 0);
+#pragma unroll 4
+    for (int i = lane; i < 5 * N; i += 32) ns[i] = __ldg(n1 + i);
+    for (int i = lane; i < 2 * (a.Np2 + a.Cp2); i += 32) ntab[i] = kFree32;  // both tables
+    __syncwarp();
+    for (int r = lane; r < N; r += 32) {
+        const float key = __ldg(n2 + (size_t)r * 5);
+        if (is_key(key)) insert32(ntab, nmask, nshift, (uint32_t)key, (uint32_t)r);
+    }
+    for (int base = 0; base < C; base += 32 * kAhead) {
+        if (base) load_rows(c2, base);
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            const int c = base + 32 * j + lane;
+            const float4 y = row[j];
+            if (!(is_key(y.x) && is_key(y.y) && !isnan(y.z))) continue;      // NaN past the last row
+            const uint32_t h = pair_hash((uint32_t)y.x, (uint32_t)y.y);
+            const uint32_t v = (h << 10) | (uint32_t)c;
+            uint32_t s = h >> cshift;
+            for (;;) {                                                       // at most half the slots are taken
+                const uint32_t old = atomicCAS(ctab + s, kFree32, v);
+                if (old == kFree32) break;
+                if ((old >> 10) == (v >> 10)) {
+                    const float4 o = __ldg(c2 + (old & 0x3ffu));
+                    if (o.x == y.x && o.y == y.y) {                          // the pair's lowest row stays
+                        atomicMin(ctab + s, v);
+                        break;
+                    }
+                }
+                s = (s + 1u) & cmask;
+            }
+        }
+    }
+    load_rows(c1, 0);
+    __syncwarp();
+    for (int base = 0; base < C; base += 32 * kAhead) {
+        if (base) load_rows(c1, base);
+        uint32_t word[kAhead];
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            const int c = base + 32 * j + lane;
+            word[j] = c < C ? __ldg(w + N + c) : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            const int c = base + 32 * j + lane;
+            float4 x = row[j];
+            if (word[j] >= 0x80000000u && is_key(x.x) && is_key(x.y) && !isnan(x.z)) {
+                const uint32_t h = pair_hash((uint32_t)x.x, (uint32_t)x.y);
+                const uint32_t bits = h & 0x3fffffu;
+                uint32_t s = h >> cshift;
+                for (;;) {
+                    const uint32_t v = ctab[s];
+                    if (v == kFree32) break;
+                    if ((v >> 10) == bits) {
+                        const float4 y = __ldg(c2 + (v & 0x3ffu));
+                        if (y.x == x.x && y.y == x.y) {
+                            x.z = y.z;
+                            x.w = y.w;
+                            break;
+                        }
+                    }
+                    s = (s + 1u) & cmask;
+                }
+            }
+            if (c < C) co[c] = x;
+        }
+    }
+    for (int r = lane; r < N; r += 32) {
+        const float key = ns[5 * r];
+        if (__ldg(w + r) >= 0x80000000u && is_key(key)) {
+            const int q = find32(ntab, nmask, nshift, (uint32_t)key);        // p2's lowest row with the key
+            if (q >= 0) {
+                const float *y = n2 + (size_t)q * 5;
+#pragma unroll
+                for (int j = 1; j < 5; ++j) ns[5 * r + j] = __ldg(y + j);
+            }
+        }
+    }
+    __syncwarp();
+#pragma unroll 4
+    for (int i = lane; i < 5 * N; i += 32) no[i] = ns[i];
+}
+
 __global__ void __launch_bounds__(kEvoThreads) crossover_kernel(const CrossArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -453,6 +870,7 @@ extern "C" int neat_mutate(float *nodes_dev, float *conns_dev, int32_t pop, neat
     a.words = words_dev;
     a.normals = normals_dev;
     a.new_keys = new_keys_dev;
+    a.pop = pop;
     a.N = d.max_nodes;
     a.C = d.max_conns;
     a.I = d.num_inputs;
@@ -489,15 +907,22 @@ extern "C" int neat_mutate(float *nodes_dev, float *conns_dev, int32_t pop, neat
     for (int i = 0; i < 8; ++i) a.act_opt[i] = m->activation_options[i];
     for (int i = 0; i < 4; ++i) a.agg_opt[i] = m->aggregation_options[i];
     a.feedforward = m->feedforward != 0;
+    if (a.N <= kWarpNodes && a.C <= kWarpConns) {
+        const int warps = pop > 4 * 152 ? 4 : 1;
+        const size_t bytes = (size_t)warps * mut_warp_layout(a.N, a.C, a.Np2).total;
+        const int rw = allow_dynamic_smem(reinterpret_cast<const void *>(mutate_warp_kernel), bytes,
+                                          "neat_mutate: shared memory");
+        if (rw) return rw;
+        mutate_warp_kernel<<<(pop + warps - 1) / warps, 32 * warps, bytes, as_stream(stream)>>>(a);
+        const cudaError_t ew = cudaGetLastError();
+        if (ew != cudaSuccess) return cuda_fail(ew, "neat_mutate: launch");
+        return NEAT_OK;
+    }
     const size_t smem = 16u * (size_t)a.Np2 + 4u * (size_t)a.N + 12u * (size_t)a.C + 4u * (size_t)a.C +
                         (size_t)a.N + 16u;
     int rc = allow_dynamic_smem(reinterpret_cast<const void *>(mutate_kernel), smem, "neat_mutate: shared memory");
     if (rc) return rc;
-    // small genomes: two warps (its block-wide steps are barrier-bound, and
-    // more genomes share an SM; 10 000 Ant-sized genomes: 0.094 -> 0.089 ms
-    // against four warps)
-    const int threads = (a.N <= 64 && a.C <= 256) ? 64 : kEvoThreads;
-    mutate_kernel<<<pop, threads, smem, as_stream(stream)>>>(a);
+    mutate_kernel<<<pop, kEvoThreads, smem, as_stream(stream)>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "neat_mutate: launch");
     return NEAT_OK;
@@ -530,11 +955,21 @@ extern "C" int neat_crossover(const float *nodes_dev, const float *conns_dev, in
     a.C = d.max_conns;
     a.Np2 = pow2_at_least(a.N);
     a.Cp2 = pow2_at_least(a.C > 0 ? a.C : 1);
+    if (a.N <= kWarpNodes && a.C <= kWarpConns) {
+        const int warps = n_children > 4 * 152 ? 4 : 1;
+        const size_t bytes = (size_t)warps * cross_warp_layout(a.N, a.Np2, a.Cp2).total;
+        const int rw = allow_dynamic_smem(reinterpret_cast<const void *>(crossover_warp_kernel), bytes,
+                                          "neat_crossover: shared memory");
+        if (rw) return rw;
+        crossover_warp_kernel<<<(n_children + warps - 1) / warps, 32 * warps, bytes, as_stream(stream)>>>(a);
+        const cudaError_t ew = cudaGetLastError();
+        if (ew != cudaSuccess) return cuda_fail(ew, "neat_crossover: launch");
+        return NEAT_OK;
+    }
     const size_t smem = 16u * ((size_t)a.Np2 + (size_t)a.Cp2);
     int rc = allow_dynamic_smem(reinterpret_cast<const void *>(crossover_kernel), smem, "neat_crossover: shared memory");
     if (rc) return rc;
-    const int threads = (a.N <= 64 && a.C <= 256) ? 128 : kEvoThreads;
-    crossover_kernel<<<n_children, threads, smem, as_stream(stream)>>>(a);
+    crossover_kernel<<<n_children, kEvoThreads, smem, as_stream(stream)>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "neat_crossover: launch");
     return NEAT_OK;

@@ -80,4 +80,41 @@ __device__ __forceinline__ int pair_row(const unsigned long long *tab, uint32_t 
     return -1;
 }
 
+// ---- the same for at most 256 rows: 32-bit entries key << 8 | row, and
+// Fibonacci hashing: the top bits of key * 2^32 / phi spread runs of
+// consecutive keys (inputs, outputs, the first hidden nodes) evenly over the
+// table, so most lookups end at their first slot.  shift = 32 - log2(slots);
+// at most half the slots are taken, so every probe sequence ends.
+constexpr uint32_t kFree32 = 0xffffffffu;
+
+__device__ __forceinline__ uint32_t slot32(uint32_t key, int shift) { return (key * 0x9E3779B1u) >> shift; }
+
+// True when the key was already present: its lowest row stays.
+__device__ __forceinline__ bool insert32(uint32_t *tab, uint32_t mask, int shift, uint32_t key, uint32_t row)
+{
+    const uint32_t v = (key << 8) | row;
+    uint32_t s = slot32(key, shift);
+    for (;;) {
+        const uint32_t old = atomicCAS(tab + s, kFree32, v);
+        if (old == kFree32) return false;
+        if ((old >> 8) == key) {
+            atomicMin(tab + s, v);
+            return true;
+        }
+        s = (s + 1u) & mask;
+    }
+}
+
+// Lowest row holding `key`, or -1.
+__device__ __forceinline__ int find32(const uint32_t *tab, uint32_t mask, int shift, uint32_t key)
+{
+    uint32_t s = slot32(key, shift);
+    for (;;) {
+        const uint32_t v = tab[s];
+        if (v == kFree32) return -1;
+        if ((v >> 8) == key) return (int)(v & 0xffu);
+        s = (s + 1u) & mask;
+    }
+}
+
 }  // namespace neat

@@ -104,6 +104,10 @@ __global__ void gen_normals_kernel(const GenDesc *__restrict__ descs, int nd)
     if (e0 >= d.count) return;
     float z[4];
     normals_of_block(d.seed, d.step, e0 >> 2, z);
+    if (e0 + 3 < d.count && (reinterpret_cast<uintptr_t>(d.out) & 15u) == 0) {
+        reinterpret_cast<float4 *>(d.out)[e0 >> 2] = make_float4(z[0], z[1], z[2], z[3]);
+        return;
+    }
     for (int k = 0; k < 4 && e0 + k < d.count; ++k) d.out[e0 + k] = z[k];
 }
 
@@ -114,6 +118,10 @@ __global__ void fill_normals_kernel(float *out, uint64_t count, uint64_t seed, i
     if (e0 >= count) return;
     float z[4];
     normals_of_block(seed, step, e0 >> 2, z);
+    if (e0 + 3 < count && (reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
+        reinterpret_cast<float4 *>(out)[e0 >> 2] = make_float4(z[0], z[1], z[2], z[3]);
+        return;
+    }
     for (int k = 0; k < 4 && e0 + k < count; ++k) out[e0 + k] = z[k];
 }
 
@@ -128,11 +136,11 @@ __global__ void gen_words_kernel(uint32_t *out, uint64_t n, uint64_t seed, uint6
                                       (uint32_t)(stream >> 32) ^ 0x574f5244u},
                                    (uint32_t)seed, (uint32_t)(seed >> 32));
         const uint64_t e = b << 2;
-        if (e + 3 < n) {
-            out[e] = r.x; out[e + 1] = r.y; out[e + 2] = r.z; out[e + 3] = r.w;
+        if (e + 3 < n && (reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
+            reinterpret_cast<uint4 *>(out)[b] = make_uint4(r.x, r.y, r.z, r.w);
         } else {
             const uint32_t v[4] = {r.x, r.y, r.z, r.w};
-            for (uint64_t k = 0; e + k < n; ++k) out[e + k] = v[k];
+            for (uint64_t k = 0; k < 4 && e + k < n; ++k) out[e + k] = v[k];
         }
     }
 }

@@ -120,7 +120,6 @@ __device__ __forceinline__ RecordOffsets record_offsets(int n, int E, int nl, in
 // 1001 genomes of 101 / 403 rows: 18 us against 29.  The bytes alone (42 MB
 // read, 19 MB written) take 9 us at the measured copy rate.
 constexpr int kWarpNodes = 128, kWarpConns = 512;
-constexpr uint32_t kFree32 = 0xffffffffu;
 
 __host__ __device__ inline int warp_record_bytes(size_t record_bytes) { return (int)((record_bytes + 15) & ~(size_t)15); }
 
@@ -142,23 +141,6 @@ __host__ __device__ inline WarpLayout warp_layout(int N, int C, int RN, int Np2)
     l.edge_of = (l.before + 2 * cw * N + 7) & ~7;                 // edges into a row from earlier connection rows
     l.total = (l.edge_of + 8 * C + 15) & ~15;                     // (rows), weight
     return l;
-}
-
-// Fibonacci hashing: the top bits of key * 2^32 / phi spread runs of
-// consecutive keys (inputs, outputs, the first hidden nodes) evenly over the
-// table, so most lookups end at their first slot.  shift = 32 - log2(slots).
-__device__ __forceinline__ uint32_t slot32(uint32_t key, int shift) { return (key * 0x9E3779B1u) >> shift; }
-
-// Lowest row holding `key`, or -1.
-__device__ __forceinline__ int find32(const uint32_t *tab, uint32_t mask, int shift, uint32_t key)
-{
-    uint32_t s = slot32(key, shift);
-    for (;;) {                               // at most half the slots are taken
-        const uint32_t v = tab[s];
-        if (v == kFree32) return -1;
-        if ((v >> 8) == key) return (int)(v & 0xffu);
-        s = (s + 1u) & mask;
-    }
 }
 
 // Connections to or from absent keys: the bit matrix cannot hold them, so
@@ -268,18 +250,7 @@ __global__ void __launch_bounds__(128) transform_warp_kernel(const TransformArgs
                     aggs |= 1u << (int)agg[i];
                 }
                 if (isnan(bias[i]) || isnan(resp[i])) st |= NEAT_G_BADATTR;
-                const uint32_t k = (uint32_t)key[i], v = (k << 8) | (uint32_t)r;
-                uint32_t s = slot32(k, kshift);
-                for (;;) {
-                    const uint32_t old = atomicCAS(ktab + s, kFree32, v);
-                    if (old == kFree32) break;
-                    if ((old >> 8) == k) {                                   // a duplicated key: its lowest row stays
-                        atomicMin(ktab + s, v);
-                        st |= NEAT_G_DUPKEY;
-                        break;
-                    }
-                    s = (s + 1u) & kmask;
-                }
+                if (insert32(ktab, kmask, kshift, (uint32_t)key[i], (uint32_t)r)) st |= NEAT_G_DUPKEY;
             }
         }
         present[i] = __ballot_sync(all, here);
