@@ -209,19 +209,6 @@ __device__ __forceinline__ void eval_node_tile(const uint4 ne, const uint2 *__re
                                         : node_output(ne, agg, act, ec, a);
 }
 
-// One whole node for one column when every non-input node of the genome
-// aggregates by sum (any activation): no aggregation dispatch.
-template <bool T1>
-__device__ __forceinline__ void eval_node_sum(const uint4 ne, const uint2 *__restrict__ edges,
-                                              float *__restrict__ v, int p, int lgT, int col)
-{
-    const uint32_t act = ne.w & 0xffu;
-    if (act == kInputAct) return;
-    const uint32_t ec = ne.z >> 16;
-    const float a = partials<T1, true>(kAggSum, edges + (ne.z & 0xffffu), ec, v, lgT, col, 0, 4);
-    v[vslot<T1>(p, lgT, col)] = activate(act, fmaf(__uint_as_float(ne.y), ec ? a : 0.0f, __uint_as_float(ne.x)));
-}
-
 // All non-input nodes of a staged record, for the columns this thread owns.
 //  Columns (T > 1): thread `lane` = (sub, col) computes column col of nodes
 //  sub, sub + nsub, ... of every level, nsub = G / T.
@@ -322,20 +309,24 @@ constexpr uint32_t kTraitsSumTanh = 1u | (0u << 8);
 __device__ __forceinline__ int ilog2(int x) { return 31 - __clz(x); }
 
 constexpr int kInputRegs = 8;   // inputs prefetched into registers per thread
+constexpr uint32_t kNoBar = 0xffffffffu;
 
 // Everything of one work item after its record copy was issued by lane 0
 // (mbarrier `bar` initialised and armed, `flag` set to 0, both before the
-// call): inputs are read into registers while the copy is in flight, the
-// group waits for the record (a bounded wait; on expiry the device error
-// word gets kErrWaitExpired and the outputs NaN), scatters the inputs into
-// the value tile, walks the levels and writes the outputs.
-//   xb: inputs of the item [bt][I]; yb: its outputs [bt][O].
+// call; bar kNoBar: the record is read where it is, nothing to wait for): inputs
+// are read into registers while the copy is in flight, the group waits for
+// the record (a bounded wait; on expiry the device error word gets
+// kErrWaitExpired and the outputs NaN), scatters the inputs into the value
+// tile, walks the levels and writes the outputs.
+//   xb: inputs of the item [bt][I]; yb: its outputs [bt][O]; vcap: floats of
+//   the value tile, at least one column of the genome's nodes (a genome with
+//   more nodes than the tile has rows takes fewer columns at a time).
 template <bool T1>
 __device__ __forceinline__ void run_item(const uint4 *srec, float *v, uint32_t bar, volatile int *flag, int G,
                                          int gi, int lane, const float *__restrict__ xb, float *__restrict__ yb,
-                                         int I, int O, int bt, int tile, int lg_split, unsigned int *err)
+                                         int I, int O, int bt, int tile, int lg_split, int vcap, unsigned int *err)
 {
-    const int lgT = T1 ? 0 : ilog2(tile);
+    int lgT = T1 ? 0 : ilog2(tile);
     const int nx = bt * I;
     float xr[kInputRegs];
 #pragma unroll
@@ -344,7 +335,7 @@ __device__ __forceinline__ void run_item(const uint4 *srec, float *v, uint32_t b
         xr[k] = (i < nx) ? __ldg(xb + i) : 0.0f;
     }
     group_sync(G, gi);                    // barrier initialised before anyone waits on it
-    if (!mbar_wait(bar, 0)) *flag = 1;
+    if (bar != kNoBar && !mbar_wait(bar, 0)) *flag = 1;
     group_sync(G, gi);
     if (*flag) {                          // uniform over the group
         if (lane == 0) atomicOr(err, kErrWaitExpired);
@@ -358,33 +349,48 @@ __device__ __forceinline__ void run_item(const uint4 *srec, float *v, uint32_t b
         return;
     }
     const uint16_t *io = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.w);
+    if constexpr (!T1)
+        while (lgT > 0 && ((int)(h0.x & 0xffffu) << lgT) > vcap) --lgT;
+    const int step = T1 ? 1 : 1 << lgT;
+    for (int c0 = 0; c0 < bt; c0 += step) {                 // once, unless the nodes outgrow the tile's rows
+        const int cols = T1 ? 1 : min(bt - c0, step);
+        const int ni = cols * I;
+        if (c0 > 0) {
+            group_sync(G, gi);                              // the last columns' outputs were read
 #pragma unroll
-    for (int k = 0; k < kInputRegs; ++k) {
-        const int i = lane + k * G;
-        if (i < nx) {
-            if (T1) v[io[i]] = xr[k];
-            else {
-                const int b = i / I, j = i - b * I;
-                v[((int)io[j] << lgT) + b] = xr[k];
+            for (int k = 0; k < kInputRegs; ++k) {
+                const int i = lane + k * G;
+                xr[k] = (i < ni) ? __ldg(xb + (size_t)c0 * I + i) : 0.0f;
             }
         }
-    }
-    for (int i = lane + kInputRegs * G; i < nx; i += G) {
-        if (T1) v[io[i]] = __ldg(xb + i);
-        else {
-            const int b = i / I, j = i - b * I;
-            v[((int)io[j] << lgT) + b] = __ldg(xb + i);
+#pragma unroll
+        for (int k = 0; k < kInputRegs; ++k) {
+            const int i = lane + k * G;
+            if (i < ni) {
+                if (T1) v[io[i]] = xr[k];
+                else {
+                    const int b = i / I, j = i - b * I;
+                    v[((int)io[j] << lgT) + b] = xr[k];
+                }
+            }
         }
-    }
-    group_sync(G, gi);
-    const bool col_ok = T1 || (lane & (tile - 1)) < bt;
-    if ((h0.w & 0xffffu) == kTraitsSumTanh) walk_levels<T1, true>(srec, v, G, gi, lane, lgT, lg_split, col_ok);
-    else walk_levels<T1, false>(srec, v, G, gi, lane, lgT, lg_split, col_ok);
-    for (int i = lane; i < bt * O; i += G) {
-        if (T1) yb[i] = v[io[I + i]];
-        else {
-            const int b = i / O, j = i - b * O;
-            yb[i] = v[((int)io[I + j] << lgT) + b];
+        for (int i = lane + kInputRegs * G; i < ni; i += G) {
+            if (T1) v[io[i]] = __ldg(xb + i);
+            else {
+                const int b = i / I, j = i - b * I;
+                v[((int)io[j] << lgT) + b] = __ldg(xb + (size_t)c0 * I + i);
+            }
+        }
+        group_sync(G, gi);
+        const bool col_ok = T1 || (lane & (step - 1)) < cols;
+        if ((h0.w & 0xffffu) == kTraitsSumTanh) walk_levels<T1, true>(srec, v, G, gi, lane, lgT, lg_split, col_ok);
+        else walk_levels<T1, false>(srec, v, G, gi, lane, lgT, lg_split, col_ok);
+        for (int i = lane; i < cols * O; i += G) {
+            if (T1) yb[i] = v[io[I + i]];
+            else {
+                const int b = i / O, j = i - b * O;
+                yb[(size_t)c0 * O + i] = v[((int)io[I + j] << lgT) + b];
+            }
         }
     }
 }

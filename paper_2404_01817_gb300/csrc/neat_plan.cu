@@ -1,11 +1,14 @@
 // Batched evaluation of several populations in one persistent launch per
 // step (the data-parallel forward of Section 3.3 over uneven populations).
 //
-// Plan creation (host, once): every record header is read back, each
-// population is split into size buckets by node count (powers of two from
-// 16), and each bucket gets a launch shape: group size G, tile T and split
-// (threads per node), chosen by a heuristic or timed on the plan's own data.
-// A bucket's work is cut into block items of `gpc` work items each
+// Every call first copies the records to compact ones, without the nodes that
+// no output depends on (compact_kernel), where that saves more than it costs.
+//
+// Plan creation (host, once): the headers of the records to be evaluated are
+// read back, each population is split into size buckets by node count (powers
+// of two from 16), and each bucket gets a launch shape: group size G, tile T
+// and split (threads per node), chosen by a heuristic or timed on the plan's
+// own data.  A bucket's work is cut into block items of `gpc` work items each
 // (gpc = threads per block / G); block items are numbered bucket by bucket,
 // largest records first, so the most expensive items start first.
 //
@@ -14,6 +17,10 @@
 // genome's record into its shared-memory region (TMA, completion on an
 // mbarrier) and then runs the same item evaluation as the single-population
 // kernel (run_item), so results match neat_forward bit for bit.
+//
+// Four populations of 2048 genomes (up to 16, 64, 256 and 1024 nodes), 64
+// inputs each: 205 us a step with compact records (509 us without), the copy
+// included.
 #include <algorithm>
 #include <climits>
 #include <cstdio>
@@ -31,6 +38,176 @@ namespace neat {
 namespace {
 
 __device__ unsigned int g_plan_error;
+
+// ---- compact records
+//
+// Nothing reads a node that reaches no output.  Before its steps, a plan
+// copies every record to a workspace of its own with only the nodes that the
+// outputs depend on (and the inputs), in the record format: positions, levels,
+// edge sources and input/output lists renumbered, every remaining node's edges
+// in their order, so its value has the same bits.  In random graphs a large
+// genome shrinks most: of 1024 node rows and 4 outputs, 23% of the nodes and
+// 12% of the edges remain, of 64 rows 54% and 44%.  The copy is made anew by
+// every call from the records as they are then; only the launch shapes come
+// from the records at creation.
+//
+// One warp per genome, straight from memory: marks the needed nodes from the
+// outputs' level down (a node's sources all lie in lower levels), ranks them
+// by population counts, writes the copy.  Bound by the latency of a chain of
+// L2 reads per level, hidden by the warps of other genomes.  (Marking inside
+// the forward kernel, by the threads that then walk the item, cost as much as
+// it saved: 541 against 509 us for the uneven plan.)
+struct CompactPop {
+    const uint8_t *src;
+    uint8_t *dst;
+    uint64_t stride;
+    int first;               // first genome's number over all populations
+    int I, O;
+};
+
+constexpr int kCompactWarps = 4;
+
+__global__ void __launch_bounds__(32 * kCompactWarps)
+compact_kernel(const CompactPop *__restrict__ pops, int np, int total, unsigned int *counters, int nc)
+{
+    __shared__ uint32_t s_bits[kCompactWarps][32];
+    __shared__ int s_pre[kCompactWarps][32];
+    __shared__ uint16_t s_list[kCompactWarps][NEAT_MAX_NODES];
+    constexpr unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (blockIdx.x == 0)                       // the steps' work counters, for the launches that follow
+        for (int i = threadIdx.x; i < nc; i += blockDim.x) counters[i] = 0u;
+    const int w = blockIdx.x * kCompactWarps + warp;
+    if (w >= total) return;
+    int lo = 0, hi = np - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (pops[mid].first <= w) lo = mid; else hi = mid - 1;
+    }
+    const CompactPop P = pops[lo];
+    const uint8_t *src = P.src + (size_t)(w - P.first) * P.stride;
+    uint8_t *dst = P.dst + (size_t)(w - P.first) * P.stride;
+    const int I = P.I, O = P.O;
+    const uint4 h0 = __ldg(reinterpret_cast<const uint4 *>(src)), h1 = __ldg(reinterpret_cast<const uint4 *>(src) + 1);
+    uint4 *out = reinterpret_cast<uint4 *>(dst);
+    if (h0.z & NEAT_G_ERROR_MASK) {
+        if (lane == 0) {
+            out[0] = h0;
+            out[1] = h1;
+        }
+        return;
+    }
+    const int n_levels = (int)(h0.x >> 16);
+    const uint4 *nodes = reinterpret_cast<const uint4 *>(src + kHeaderBytes);
+    const uint2 *edges = reinterpret_cast<const uint2 *>(src + h1.y);
+    const uint16_t *lev = reinterpret_cast<const uint16_t *>(src + h1.z);
+    const uint16_t *io = reinterpret_cast<const uint16_t *>(src + h1.w);
+    uint32_t *bits = s_bits[warp];
+    int *pre = s_pre[warp];
+    uint16_t *list = s_list[warp];
+    bits[lane] = 0u;
+    __syncwarp();
+    int last = 0;
+    for (int j = lane; j < O; j += 32) {
+        const int p = __ldg(io + I + j);
+        last = max(last, p);
+        atomicOr(bits + (p >> 5), 1u << (p & 31));
+    }
+    last = __reduce_max_sync(all, last);
+    __syncwarp();
+    int top = n_levels - 1;
+    while ((int)__ldg(lev + top) > last) --top;                // the levels above every output
+    for (int l = top; l > 0; --l) {
+        const int p1 = __ldg(lev + l + 1);
+        for (int p = __ldg(lev + l) + lane; p < p1; p += 32) {
+            if (!((bits[p >> 5] >> (p & 31)) & 1u)) continue;
+            const uint32_t z = __ldg(&nodes[p].z);
+            const int b = (int)(z & 0xffffu), e = b + (int)(z >> 16);
+            for (int i = b; i < e; i += 4) {
+                uint32_t s[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) s[k] = i + k < e ? __ldg(&edges[i + k].y) : all;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (s[k] != all) atomicOr(bits + (s[k] >> 5), 1u << (s[k] & 31u));
+            }
+        }
+        __syncwarp();
+    }
+    for (int j = lane; j < I; j += 32) {
+        const int p = __ldg(io + j);
+        atomicOr(bits + (p >> 5), 1u << (p & 31));
+    }
+    __syncwarp();
+    const uint32_t mine = bits[lane];
+    int incl = __popc(mine);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(all, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int n = __shfl_sync(all, incl, 31);
+    pre[lane] = incl - __popc(mine);
+    {
+        int k = incl - __popc(mine);
+        for (uint32_t m = mine; m; m &= m - 1u) list[k++] = (uint16_t)(32 * lane + __ffs(m) - 1);
+    }
+    __syncwarp();
+    auto rank = [&](uint32_t p) { return (uint32_t)(pre[p >> 5] + __popc(bits[p >> 5] & ((1u << (p & 31u)) - 1u))); };
+    const uint32_t off_edge = kHeaderBytes + kNodeBytes * (uint32_t)n;
+    uint2 *edges_out = reinterpret_cast<uint2 *>(dst + off_edge);
+    int carry = 0;
+    unsigned lead = (unsigned)n;                               // leading positions that are inputs
+    for (int k0 = 0; k0 < n; k0 += 32) {
+        const int k = k0 + lane;
+        uint4 ne = make_uint4(0u, 0u, 0u, (uint32_t)kInputAct);
+        if (k < n) ne = __ldg(nodes + list[k]);
+        const int ec = (int)(ne.z >> 16), b = (int)(ne.z & 0xffffu);
+        int sum = ec;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(all, sum, o);
+            if (lane >= o) sum += y;
+        }
+        const int to = carry + sum - ec;
+        carry += __shfl_sync(all, sum, 31);
+        if (k >= n) continue;
+        if ((ne.w & 0xffu) != kInputAct) lead = min(lead, (unsigned)k);
+        out[2 + k] = make_uint4(ne.x, ne.y, (uint32_t)to | ((uint32_t)ec << 16), ne.w);
+        for (int i = 0; i < ec; i += 4) {
+            uint2 e[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i + q < ec) e[q] = __ldg(edges + b + i + q);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i + q < ec) edges_out[to + i + q] = make_uint2(e[q].x, rank(e[q].y));
+        }
+    }
+    lead = __reduce_min_sync(all, lead);
+    const uint32_t off_level = align16(off_edge + kEdgeBytes * (uint32_t)carry);
+    const uint32_t off_io = align16(off_level + 2u * (uint32_t)(top + 2));
+    uint16_t *lev_out = reinterpret_cast<uint16_t *>(dst + off_level);
+    for (int l = lane; l <= top; l += 32) lev_out[l] = (uint16_t)rank(__ldg(lev + l));
+    uint16_t *io_out = reinterpret_cast<uint16_t *>(dst + off_io);
+    for (int j = lane; j < I + O; j += 32) io_out[j] = (uint16_t)rank(__ldg(io + j));
+    if (lane == 0) {
+        lev_out[top + 1] = (uint16_t)n;
+        out[0] = make_uint4((uint32_t)n | ((uint32_t)(top + 1) << 16), (uint32_t)carry, h0.z,
+                            (h0.w & 0xffffu) | (lead << 16));
+        out[1] = make_uint4(align16(off_io + 2u * (uint32_t)(I + O)), off_edge, off_level, off_io);
+    }
+}
+
+// An item whose record or nodes outgrow its group's region (a record changed
+// since the plan chose its shapes): read where it lies.
+template <bool T1>
+__device__ __noinline__ void run_item_in_place(const uint4 *rec, float *v, volatile int *flag, int G, int gi, int lane,
+                                               const float *xb, float *yb, int I, int O, int bt, int tile, int lg_split,
+                                               int vcap, unsigned int *err)
+{
+    run_item<T1>(rec, v, kNoBar, flag, G, gi, lane, xb, yb, I, O, bt, tile, lg_split, vcap, err);
+}
 
 template <bool PDL>
 __global__ void __launch_bounds__(1024, 1)
@@ -62,16 +239,25 @@ plan_kernel(const BucketDev *__restrict__ buckets, int nb, int item_lo, int item
         uint4 *srec = regions + (size_t)gi * d.region_words;
         const uint32_t bar = smem_addr(bars + gi);
         int g = 0, b0 = 0;
+        bool staged = true;
         if (active) {
             const int k = (int)(item / d.tiles);
             g = __ldg(d.gidx + k);
             b0 = (int)(item - (long)k * d.tiles) * d.tile;
+            const uint8_t *grec = d.rec + (size_t)g * d.stride;
+            uint32_t bytes = (uint32_t)d.rec_copy_bytes;
+            if (bytes == 0) {                          // a compact record's own size
+                bytes = align16(__ldg(reinterpret_cast<const uint32_t *>(grec) + 4));
+                staged = bytes <= (uint32_t)d.rec_words * 16u;
+            }
             if (lane == 0) {
                 flags[gi] = 0;
-                fence_proxy_async_smem();              // the region was read by the previous item
-                mbar_init(bar, 1);
-                mbar_arrive_expect_tx(bar, (uint32_t)d.rec_copy_bytes);
-                bulk_g2s(smem_addr(srec), d.rec + (size_t)g * d.stride, (uint32_t)d.rec_copy_bytes, bar);
+                if (staged) {
+                    fence_proxy_async_smem();          // the region was read by the previous item
+                    mbar_init(bar, 1);
+                    mbar_arrive_expect_tx(bar, bytes);
+                    bulk_g2s(smem_addr(srec), grec, bytes, bar);
+                }
             }
         }
         if (PDL && !waited) {                          // inputs of this step may come from the previous kernel
@@ -84,13 +270,25 @@ plan_kernel(const BucketDev *__restrict__ buckets, int nb, int item_lo, int item
             const float *xb = d.x + d.x_step * step + ((size_t)g * d.B + b0) * d.I;
             float *yb = d.y + d.y_step * step + ((size_t)g * d.B + b0) * d.O;
             float *v = reinterpret_cast<float *>(srec + d.rec_words);
-            if (d.tile == 1)
-                run_item<true>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split, &g_plan_error);
-            else
-                run_item<false>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, &g_plan_error);
+            const int vcap = (d.region_words - d.rec_words) * 4;
+            if (!staged) {
+                const uint4 *grec = reinterpret_cast<const uint4 *>(d.rec + (size_t)g * d.stride);
+                if (d.tile == 1)
+                    run_item_in_place<true>(grec, v, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split, vcap,
+                                            &g_plan_error);
+                else
+                    run_item_in_place<false>(grec, v, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, vcap,
+                                             &g_plan_error);
+            } else if (d.tile == 1) {
+                run_item<true>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split, vcap,
+                               &g_plan_error);
+            } else {
+                run_item<false>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, vcap,
+                                &g_plan_error);
+            }
         }
         __syncthreads();
-        if (active && lane == 0) mbar_inval(bar);      // re-initialised by the next item using this slot
+        if (active && staged && lane == 0) mbar_inval(bar);   // re-initialised by the next item using this slot
     }
 }
 
@@ -102,6 +300,7 @@ struct HostBucket {
     int pop_index = 0;
     int n_class = 0;         // node-count bound of the bucket
     int max_used = 0;        // largest record (bytes) in the bucket
+    int max_rows = 0;        // value tile rows: most nodes of a record in the bucket
     std::vector<int32_t> gidx;
     Shape shape;
 };
@@ -166,18 +365,35 @@ struct neat_plan {
     std::string autotune_log;
     int max_footprint_bucket = -1;    // host bucket whose groups take the most shared memory
     size_t smem_override = 0;         // while timing one bucket: its own footprint
+    uint8_t *d_compact = nullptr;     // compact records (null: the records themselves are evaluated)
+    CompactPop *d_cpops = nullptr;
+    std::vector<uint8_t *> compact_of;   // by population
+    int n_cpops = 0, n_genomes = 0;
 };
 
 namespace neat {
 namespace {
 
-size_t region_bytes(const HostBucket &b, int I, int O)
+size_t region_bytes(const neat_plan *P, const HostBucket &b)
 {
-    (void)I;
-    (void)O;
     const size_t rec = (size_t)align16((uint32_t)b.max_used);
-    const size_t vals = 4u * (size_t)((b.n_class * b.shape.tile + 3) & ~3);
-    return (rec + vals + 15) & ~(size_t)15;
+    // one column of any genome of the population fits, whatever its record
+    // becomes (run_item takes fewer columns at a time then)
+    const int vals = std::max(b.max_rows * b.shape.tile, P->pops[b.pop_index].dims.max_nodes);
+    return (rec + 4u * (size_t)((vals + 3) & ~3) + 15) & ~(size_t)15;
+}
+
+// Compact records from the records as they are now, and `counters` cleared.
+int launch_compact(neat_plan *P, int counters, cudaStream_t s)
+{
+    if (!P->d_compact) {
+        const cudaError_t e = cudaMemsetAsync(P->d_counters, 0, sizeof(unsigned int) * (size_t)counters, s);
+        return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "plan: counter reset");
+    }
+    const int blocks = (P->n_genomes + kCompactWarps - 1) / kCompactWarps;
+    compact_kernel<<<blocks, 32 * kCompactWarps, 0, s>>>(P->d_cpops, P->n_cpops, P->n_genomes, P->d_counters, counters);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "plan: compact launch");
 }
 
 // Lay out the block items and the device bucket table for the current shapes.
@@ -205,7 +421,7 @@ int layout(neat_plan *P, cudaStream_t s)
         const HostBucket &h = P->hb[bi];
         const neat_pop_desc &pd = P->pops[h.pop_index];
         BucketDev d;
-        d.rec = static_cast<const uint8_t *>(pd.transformed_dev);
+        d.rec = P->d_compact ? P->compact_of[h.pop_index] : static_cast<const uint8_t *>(pd.transformed_dev);
         d.gidx = P->d_gidx + goffs[bi];
         d.x = pd.inputs_dev;
         d.y = pd.outputs_dev;
@@ -222,7 +438,7 @@ int layout(neat_plan *P, cudaStream_t s)
         if (!shape_ok(h.shape, NT)) return invalid("plan: invalid bucket launch shape");
         d.G = h.shape.G;
         d.lgG = lg(d.G);
-        const size_t reg = region_bytes(h, d.I, d.O);
+        const size_t reg = region_bytes(P, h);
         int gpc = NT / d.G;
         if (d.G > 32) gpc = std::min(gpc, 15);
         while (gpc > 1 && reg * gpc > 200u * 1024u) --gpc;
@@ -231,7 +447,7 @@ int layout(neat_plan *P, cudaStream_t s)
         d.gpc = gpc;
         d.region_words = (int)(reg / 16);
         d.rec_words = (int)(align16((uint32_t)h.max_used) / 16);
-        d.rec_copy_bytes = (int)align16((uint32_t)h.max_used);
+        d.rec_copy_bytes = P->d_compact ? 0 : (int)align16((uint32_t)h.max_used);
         const long items = (long)d.n_genomes * d.tiles;
         d.cta_begin = cta;
         d.cta_items = (int)((items + gpc - 1) / gpc);
@@ -402,7 +618,7 @@ size_t footprint(const neat_plan *P, const HostBucket &h)
 {
     int gpc = P->block_threads / h.shape.G;
     if (h.shape.G > 32) gpc = std::min(gpc, 15);
-    return region_bytes(h, 0, 0) * gpc;
+    return region_bytes(P, h) * gpc;
 }
 
 int autotune(neat_plan *P, cudaStream_t s, float *step_ms)
@@ -518,6 +734,92 @@ int autotune_block_threads(neat_plan *P, cudaStream_t s)
     return layout(P, s);
 }
 
+// The workspace of the compact records, and a first copy.  Without memory for
+// it the plan evaluates the records themselves.
+int make_compact(neat_plan *P, cudaStream_t s)
+{
+    size_t bytes = 0;
+    std::vector<CompactPop> cp;
+    std::vector<int> order(P->pops.size());
+    P->compact_of.assign(P->pops.size(), nullptr);
+    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+    // the largest records' long chains first
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return record_stride(P->pops[a].dims) > record_stride(P->pops[b].dims);
+    });
+    for (const neat_pop_desc &pd : P->pops)
+        if (pd.pop > 0 && pd.batch > 0) bytes += record_stride(pd.dims) * (size_t)pd.pop;
+    if (bytes == 0) return NEAT_OK;
+    if (cudaMalloc(&P->d_compact, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        P->d_compact = nullptr;
+        return NEAT_OK;
+    }
+    size_t off = 0;
+    for (int p : order) {
+        const neat_pop_desc &pd = P->pops[p];
+        if (pd.pop == 0 || pd.batch == 0) continue;
+        CompactPop c;
+        c.src = static_cast<const uint8_t *>(pd.transformed_dev);
+        c.dst = P->compact_of[p] = P->d_compact + off;
+        c.stride = record_stride(pd.dims);
+        c.first = P->n_genomes;
+        c.I = pd.dims.num_inputs;
+        c.O = pd.dims.num_outputs;
+        off += c.stride * (size_t)pd.pop;
+        P->n_genomes += pd.pop;
+        cp.push_back(c);
+    }
+    P->n_cpops = (int)cp.size();
+    cudaError_t e = cudaMalloc(&P->d_cpops, sizeof(CompactPop) * cp.size());
+    if (e != cudaSuccess) return cuda_fail(e, "neat_plan_create: cudaMalloc");
+    e = cudaMemcpyAsync(P->d_cpops, cp.data(), sizeof(CompactPop) * cp.size(), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return cuda_fail(e, "neat_plan_create: copy");
+    const int rc = launch_compact(P, 1, s);
+    if (rc) return rc;
+    e = cudaStreamSynchronize(s);              // cp goes out of scope
+    return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "neat_plan_create: synchronize");
+}
+
+void free_compact(neat_plan *P)
+{
+    if (P->d_compact) cudaFree(P->d_compact);
+    if (P->d_cpops) cudaFree(P->d_cpops);
+    P->d_compact = nullptr;
+    P->d_cpops = nullptr;
+}
+
+int read_headers(neat_plan *P, bool compact, cudaStream_t s, std::vector<std::vector<uint32_t>> *out)
+{
+    out->assign(P->pops.size(), {});
+    for (size_t p = 0; p < P->pops.size(); ++p) {
+        const neat_pop_desc &pd = P->pops[p];
+        if (pd.pop == 0 || pd.batch == 0) continue;
+        (*out)[p].resize((size_t)pd.pop * 8);
+        const void *src = compact ? P->compact_of[p] : pd.transformed_dev;
+        const cudaError_t e = cudaMemcpy2DAsync((*out)[p].data(), 32, src, record_stride(pd.dims), 32, (size_t)pd.pop,
+                                                cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) return cuda_fail(e, "neat_plan_create: header copy");
+    }
+    return NEAT_OK;
+}
+
+// Whether the nodes saved are worth the copy that every call makes: a warp's
+// work on one node for 32 columns is about 130 instructions, so the 8 us or
+// so that the copy takes are 50 000 of them at the rate the steps run at.
+bool compact_pays(const neat_plan *P, const std::vector<std::vector<uint32_t>> &full,
+                  const std::vector<std::vector<uint32_t>> &compact)
+{
+    double saved = 0.0;
+    for (size_t p = 0; p < full.size(); ++p) {
+        const int batch = P->pops[p].batch;
+        const double per_node = batch <= 1 ? 0.25 : (double)((batch + 31) / 32);
+        for (size_t g = 0; g * 8 < full[p].size(); ++g)
+            saved += per_node * ((double)(full[p][g * 8] & 0xffffu) - (double)(compact[p][g * 8] & 0xffffu));
+    }
+    return saved > 50000.0;
+}
+
 }  // namespace
 }  // namespace neat
 
@@ -550,23 +852,21 @@ extern "C" int neat_plan_create(const neat_pop_desc *pops, int32_t npops, const 
     P->pops.assign(pops, pops + npops);
     P->opt = o;
     P->block_threads = o.block_threads;
-    // read every header once
-    std::vector<std::vector<uint32_t>> hdrs(npops);
-    for (int p = 0; p < npops; ++p) {
-        const neat_pop_desc &pd = pops[p];
-        if (pd.pop == 0 || pd.batch == 0) continue;
-        hdrs[p].resize((size_t)pd.pop * 8);
-        cudaError_t e = cudaMemcpy2DAsync(hdrs[p].data(), 32, pd.transformed_dev, record_stride(pd.dims), 32,
-                                          (size_t)pd.pop, cudaMemcpyDeviceToHost, s);
-        if (e != cudaSuccess) {
-            delete P;
-            return cuda_fail(e, "neat_plan_create: header copy");
-        }
+    // read every header once, and those of the compact records
+    std::vector<std::vector<uint32_t>> hdrs, chdrs;
+    int rc = ensure_counters(P, 1);
+    if (rc == NEAT_OK) rc = make_compact(P, s);
+    if (rc == NEAT_OK) rc = read_headers(P, false, s, &hdrs);
+    if (rc == NEAT_OK && P->d_compact) rc = read_headers(P, true, s, &chdrs);
+    cudaError_t e = cudaSuccess;
+    if (rc == NEAT_OK && (e = cudaStreamSynchronize(s)) != cudaSuccess) rc = cuda_fail(e, "neat_plan_create: synchronize");
+    if (rc != NEAT_OK) {
+        neat_plan_destroy(P);
+        return rc;
     }
-    cudaError_t e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) {
-        delete P;
-        return cuda_fail(e, "neat_plan_create: synchronize");
+    if (P->d_compact) {
+        if (compact_pays(P, hdrs, chdrs)) hdrs.swap(chdrs);
+        else free_compact(P);
     }
     for (int p = 0; p < npops; ++p) {
         const neat_pop_desc &pd = pops[p];
@@ -589,6 +889,7 @@ extern "C" int neat_plan_create(const neat_pop_desc *pops, int32_t npops, const 
             }
             HostBucket &b = P->hb[slot_of_class[key]];
             b.gidx.push_back(g);
+            b.max_rows = P->d_compact ? std::max(b.max_rows, n) : b.n_class;
             const uint32_t used = std::min<uint32_t>(h[4], record_max_bytes(pd.dims.num_inputs, pd.dims.num_outputs,
                                                                             pd.dims.max_nodes, pd.dims.max_conns));
             b.max_used = std::max<int>(b.max_used, (int)align16(used));
@@ -611,7 +912,7 @@ extern "C" int neat_plan_create(const neat_pop_desc *pops, int32_t npops, const 
     if (total > 0) {
         e = cudaMalloc(&P->d_gidx, sizeof(int32_t) * total);
         if (e != cudaSuccess) {
-            delete P;
+            neat_plan_destroy(P);
             return cuda_fail(e, "neat_plan_create: cudaMalloc indices");
         }
         size_t off = 0;
@@ -625,8 +926,7 @@ extern "C" int neat_plan_create(const neat_pop_desc *pops, int32_t npops, const 
             off += b.gidx.size();
         }
     }
-    int rc = ensure_counters(P, 1);
-    if (rc == NEAT_OK) rc = layout(P, s);
+    rc = layout(P, s);
     if (rc == NEAT_OK && o.autotune && !P->hb.empty())
         rc = tune_block ? autotune_block_threads(P, s) : autotune(P, s, nullptr);
     if (rc == NEAT_OK) {
@@ -649,8 +949,8 @@ extern "C" int neat_plan_forward(neat_plan *P, int32_t step, void *stream)
     if (step < 0) return invalid("neat_plan_forward: step < 0");
     if (P->total_items == 0) return NEAT_OK;
     cudaStream_t s = as_stream(stream);
-    cudaError_t e = cudaMemsetAsync(P->d_counters, 0, sizeof(unsigned int), s);
-    if (e != cudaSuccess) return cuda_fail(e, "neat_plan_forward: counter reset");
+    const int rc = launch_compact(P, 1, s);
+    if (rc) return rc;
     return launch_step(P, 0, P->total_items, P->d_counters, step, false, s);
 }
 
@@ -675,15 +975,15 @@ extern "C" int neat_plan_forward_steps(neat_plan *P, int32_t first_step, int32_t
         }
         e = cudaStreamBeginCapture(P->cap, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(e, "neat_plan_forward_steps: begin capture");
-        e = cudaMemsetAsync(P->d_counters, 0, sizeof(unsigned int) * (size_t)steps, P->cap);
-        for (int k = 0; k < steps && rc == NEAT_OK && e == cudaSuccess; ++k)
+        rc = launch_compact(P, steps, P->cap);
+        for (int k = 0; k < steps && rc == NEAT_OK; ++k)
             rc = launch_step(P, 0, P->total_items, P->d_counters + k, first_step + k, P->opt.pdl && k > 0, P->cap);
         cudaGraph_t graph = nullptr;
         cudaError_t e2 = cudaStreamEndCapture(P->cap, &graph);
-        if (rc != NEAT_OK || e != cudaSuccess || e2 != cudaSuccess) {
+        if (rc != NEAT_OK || e2 != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
             if (rc) return rc;
-            return cuda_fail(e != cudaSuccess ? e : e2, "neat_plan_forward_steps: capture");
+            return cuda_fail(e2, "neat_plan_forward_steps: capture");
         }
         e = cudaGraphInstantiate(&P->exec, graph, 0);
         cudaGraphDestroy(graph);
@@ -711,7 +1011,7 @@ extern "C" int neat_plan_describe(const neat_plan *P, char *buf, int32_t len)
         snprintf(tmp, sizeof(tmp),
                  "%s{\"genomes\":%d,\"batch\":%d,\"G\":%d,\"tile\":%d,\"split\":%d,\"groups_per_block\":%d,"
                  "\"record_bytes\":%d,\"region_bytes\":%d,\"block_items\":%d}",
-                 i ? "," : "", d.n_genomes, d.B, d.G, d.tile, 1 << d.lg_split, d.gpc, d.rec_copy_bytes,
+                 i ? "," : "", d.n_genomes, d.B, d.G, d.tile, 1 << d.lg_split, d.gpc, d.rec_words * 16,
                  d.region_words * 16, d.cta_items);
         js += tmp;
     }
@@ -732,6 +1032,7 @@ extern "C" void neat_plan_destroy(neat_plan *P)
     if (P->d_buckets) cudaFree(P->d_buckets);
     if (P->d_gidx) cudaFree(P->d_gidx);
     if (P->d_counters) cudaFree(P->d_counters);
+    free_compact(P);
     delete P;
 }
 
