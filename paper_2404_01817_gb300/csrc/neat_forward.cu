@@ -324,6 +324,10 @@ int choose_groups_per_block(long items, int group, size_t per_group, const Devic
     int best = 1;
     long best_waves = -1, best_load = -1;
     for (int gpb = 1; gpb <= max_gpb; ++gpb) {
+        // a block's groups are a lower bound of the load: nothing beyond one
+        // wave's best load can match it (256 tries become 2 for 100 genomes of
+        // 4 threads, several microseconds of a call that takes ten)
+        if (best_waves == 1 && gpb > best_load) break;
         const size_t smem = per_group * gpb + 16u * (size_t)forward_header_words(gpb);
         if (smem > 227u * 1024u) break;
         const int threads = group * gpb;

@@ -213,7 +213,9 @@ def _check(code: int, where: str) -> None:
 def _stream(stream) -> int | None:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        # the handle of torch.cuda.current_stream() without the Stream object
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
     return getattr(stream, "cuda_stream", stream)
 
 
@@ -268,10 +270,9 @@ def neat_transform(nodes, conns, d: Dims, transformed=None, status=None, stream=
     pop = nodes.shape[0]
     assert nodes.is_cuda and nodes.dtype == torch.float32 and nodes.is_contiguous()
     assert conns.is_cuda and conns.dtype == torch.float32 and conns.is_contiguous()
-    assert tuple(nodes.shape[1:]) == (d.max_nodes, 5) and tuple(conns.shape[1:]) == (d.max_conns, 4)
-    nbytes = neat_transformed_bytes(pop, d)
+    assert nodes.shape[1:] == (d.max_nodes, 5) and conns.shape[1:] == (d.max_conns, 4)
     if transformed is None:
-        transformed = torch.empty(max(nbytes, 16), dtype=torch.uint8, device=nodes.device)
+        transformed = torch.empty(max(neat_transformed_bytes(pop, d), 16), dtype=torch.uint8, device=nodes.device)
     if status is None:
         status = torch.empty(max(pop, 1), dtype=torch.int32, device=nodes.device)
     _check(_lib.neat_transform(_ptr(nodes), _ptr(conns), pop, d, _ptr(transformed),
@@ -285,9 +286,8 @@ def neat_transform_recurrent(nodes, conns, d: Dims, transformed=None, status=Non
     import torch
     pop = nodes.shape[0]
     assert nodes.is_cuda and conns.is_cuda and nodes.is_contiguous() and conns.is_contiguous()
-    nbytes = neat_transformed_bytes(pop, d)
     if transformed is None:
-        transformed = torch.empty(max(nbytes, 16), dtype=torch.uint8, device=nodes.device)
+        transformed = torch.empty(max(neat_transformed_bytes(pop, d), 16), dtype=torch.uint8, device=nodes.device)
     if status is None:
         status = torch.empty(max(pop, 1), dtype=torch.int32, device=nodes.device)
     _check(_lib.neat_transform_recurrent(_ptr(nodes), _ptr(conns), pop, d, _ptr(transformed),
