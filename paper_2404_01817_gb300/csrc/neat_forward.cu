@@ -78,7 +78,8 @@ __global__ void __launch_bounds__(1024, 1) forward_kernel(const ForwardArgs a)
         pdl_trigger();
     }
     run_item<T1>(srec, v, bar, flags + gi, G, gi, lane, a.x + ((size_t)g * a.B + b0) * a.I,
-                 a.y + ((size_t)g * a.B + b0) * a.O, a.I, a.O, bt, a.tile, a.lg_split, a.val_floats, &g_forward_error);
+                 a.y + ((size_t)g * a.B + b0) * a.O, a.I, a.O, bt, a.tile, a.lg_split, a.val_floats, 0xffffffffu,
+                 &g_forward_error);
 }
 
 // One thread per genome (group 1, tile 1): each thread walks the positions

@@ -116,9 +116,17 @@ struct BucketDev {
 };
 
 // A whole population as one bucket with the heuristic launch shape; gidx_dev
-// must list genomes 0..pop-1.  *footprint: shared memory of its groups.
+// must list genomes 0..pop-1.  own_size: each record's copy is as long as its
+// header says.  max_used, max_rows: no record is longer or has more nodes (0:
+// what the dims allow).  *footprint: shared memory of its groups.
 int fill_population_bucket(const neat_pop_desc &pd, const int32_t *gidx_dev, int block_threads, int cta_begin,
-                           BucketDev *out, size_t *footprint);
+                           BucketDev *out, size_t *footprint, bool own_size = false, int max_used = 0,
+                           int max_rows = 0);
+// Copies of a population's records without the nodes that no output depends
+// on (neat_plan.cu), at the same stride.  largest_dev (may be NULL): two words,
+// raised to the most bytes and the most nodes of a copy.
+int launch_compact_population(const void *src, void *dst, int pop, const neat_dims &d, unsigned int *largest_dev,
+                              cudaStream_t s);
 // Launch the persistent kernel over a bucket table already in device memory
 // (counter_dev must be zero).
 int launch_plan_table(const BucketDev *table_dev, int nb, int total_items, unsigned int *counter_dev, int step,

@@ -321,10 +321,13 @@ constexpr uint32_t kNoBar = 0xffffffffu;
 //   xb: inputs of the item [bt][I]; yb: its outputs [bt][O]; vcap: floats of
 //   the value tile, at least one column of the genome's nodes (a genome with
 //   more nodes than the tile has rows takes fewer columns at a time).
+// False, with nothing evaluated, when the record is longer than rec_limit
+// bytes (the part that was copied).
 template <bool T1>
-__device__ __forceinline__ void run_item(const uint4 *srec, float *v, uint32_t bar, volatile int *flag, int G,
+__device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t bar, volatile int *flag, int G,
                                          int gi, int lane, const float *__restrict__ xb, float *__restrict__ yb,
-                                         int I, int O, int bt, int tile, int lg_split, int vcap, unsigned int *err)
+                                         int I, int O, int bt, int tile, int lg_split, int vcap, uint32_t rec_limit,
+                                         unsigned int *err)
 {
     int lgT = T1 ? 0 : ilog2(tile);
     const int nx = bt * I;
@@ -341,13 +344,14 @@ __device__ __forceinline__ void run_item(const uint4 *srec, float *v, uint32_t b
         if (lane == 0) atomicOr(err, kErrWaitExpired);
         mbar_wait(bar, 0);                // let the copy land before the region is reused
         for (int i = lane; i < bt * O; i += G) yb[i] = __int_as_float(0x7fc00000);
-        return;
+        return true;
     }
     const uint4 h0 = srec[0], h1 = srec[1];
     if (h0.z & NEAT_G_ERROR_MASK) {
         for (int i = lane; i < bt * O; i += G) yb[i] = __int_as_float(0x7fc00000);
-        return;
+        return true;
     }
+    if (h1.x > rec_limit) return false;
     const uint16_t *io = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.w);
     if constexpr (!T1)
         while (lgT > 0 && ((int)(h0.x & 0xffffu) << lgT) > vcap) --lgT;
@@ -393,6 +397,7 @@ __device__ __forceinline__ void run_item(const uint4 *srec, float *v, uint32_t b
             }
         }
     }
+    return true;
 }
 
 }  // namespace neat

@@ -19,8 +19,8 @@
 // kernel (run_item), so results match neat_forward bit for bit.
 //
 // Four populations of 2048 genomes (up to 16, 64, 256 and 1024 nodes), 64
-// inputs each: 205 us a step with compact records (509 us without), the copy
-// included.
+// inputs each: 189 us a step with compact records (509 us without), the 49 us
+// copy included.
 #include <algorithm>
 #include <climits>
 #include <cstdio>
@@ -52,9 +52,9 @@ __device__ unsigned int g_plan_error;
 // from the records at creation.
 //
 // One warp per genome, straight from memory: marks the needed nodes from the
-// outputs' level down (a node's sources all lie in lower levels), ranks them
-// by population counts, writes the copy.  Bound by the latency of a chain of
-// L2 reads per level, hidden by the warps of other genomes.  (Marking inside
+// outputs back, ranks them by population counts, writes the copy.  Bound by
+// the latency of a chain of L2 reads per round, hidden by the warps of other
+// genomes.  (Marking inside
 // the forward kernel, by the threads that then walk the item, cost as much as
 // it saved: 541 against 509 us for the uneven plan.)
 struct CompactPop {
@@ -68,7 +68,8 @@ struct CompactPop {
 constexpr int kCompactWarps = 4;
 
 __global__ void __launch_bounds__(32 * kCompactWarps)
-compact_kernel(const CompactPop *__restrict__ pops, int np, int total, unsigned int *counters, int nc)
+compact_kernel(const CompactPop *__restrict__ pops, int np, const CompactPop one, int total, unsigned int *counters,
+               int nc, unsigned int *largest)
 {
     __shared__ uint32_t s_bits[kCompactWarps][32];
     __shared__ int s_pre[kCompactWarps][32];
@@ -84,7 +85,7 @@ compact_kernel(const CompactPop *__restrict__ pops, int np, int total, unsigned 
         const int mid = (lo + hi + 1) >> 1;
         if (pops[mid].first <= w) lo = mid; else hi = mid - 1;
     }
-    const CompactPop P = pops[lo];
+    const CompactPop P = np > 0 ? pops[lo] : one;
     const uint8_t *src = P.src + (size_t)(w - P.first) * P.stride;
     uint8_t *dst = P.dst + (size_t)(w - P.first) * P.stride;
     const int I = P.I, O = P.O;
@@ -115,25 +116,40 @@ compact_kernel(const CompactPop *__restrict__ pops, int np, int total, unsigned 
     }
     last = __reduce_max_sync(all, last);
     __syncwarp();
-    int top = n_levels - 1;
-    while ((int)__ldg(lev + top) > last) --top;                // the levels above every output
-    for (int l = top; l > 0; --l) {
-        const int p1 = __ldg(lev + l + 1);
-        for (int p = __ldg(lev + l) + lane; p < p1; p += 32) {
-            if (!((bits[p >> 5] >> (p & 31)) & 1u)) continue;
-            const uint32_t z = __ldg(&nodes[p].z);
+    // from the outputs back, a round for all nodes marked since the last one:
+    // a node each lane, whatever its level (rounds of one level each leave
+    // most lanes idle)
+    uint32_t done = 0u;                                        // of word `lane`
+    for (;;) {
+        const uint32_t fresh = bits[lane] & ~done;
+        done |= fresh;
+        int incl = __popc(fresh);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(all, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int count = __shfl_sync(all, incl, 31);
+        if (count == 0) break;
+        int k = incl - __popc(fresh);
+        for (uint32_t m = fresh; m; m &= m - 1u) list[k++] = (uint16_t)(32 * lane + __ffs(m) - 1);
+        __syncwarp();
+        for (int q = lane; q < count; q += 32) {
+            const uint32_t z = __ldg(&nodes[list[q]].z);
             const int b = (int)(z & 0xffffu), e = b + (int)(z >> 16);
             for (int i = b; i < e; i += 4) {
                 uint32_t s[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) s[k] = i + k < e ? __ldg(&edges[i + k].y) : all;
+                for (int k4 = 0; k4 < 4; ++k4) s[k4] = i + k4 < e ? __ldg(&edges[i + k4].y) : all;
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (s[k] != all) atomicOr(bits + (s[k] >> 5), 1u << (s[k] & 31u));
+                for (int k4 = 0; k4 < 4; ++k4)
+                    if (s[k4] != all) atomicOr(bits + (s[k4] >> 5), 1u << (s[k4] & 31u));
             }
         }
         __syncwarp();
     }
+    int top = n_levels - 1;
+    while ((int)__ldg(lev + top) > last) --top;                // the levels above every output
     for (int j = lane; j < I; j += 32) {
         const int p = __ldg(io + j);
         atomicOr(bits + (p >> 5), 1u << (p & 31));
@@ -195,7 +211,12 @@ compact_kernel(const CompactPop *__restrict__ pops, int np, int total, unsigned 
         lev_out[top + 1] = (uint16_t)n;
         out[0] = make_uint4((uint32_t)n | ((uint32_t)(top + 1) << 16), (uint32_t)carry, h0.z,
                             (h0.w & 0xffffu) | (lead << 16));
-        out[1] = make_uint4(align16(off_io + 2u * (uint32_t)(I + O)), off_edge, off_level, off_io);
+        const uint32_t used = align16(off_io + 2u * (uint32_t)(I + O));
+        out[1] = make_uint4(used, off_edge, off_level, off_io);
+        if (largest) {                                         // most bytes and nodes of a copy
+            atomicMax(largest, used);
+            atomicMax(largest + 1, (unsigned int)n);
+        }
     }
 }
 
@@ -206,7 +227,7 @@ __device__ __noinline__ void run_item_in_place(const uint4 *rec, float *v, volat
                                                const float *xb, float *yb, int I, int O, int bt, int tile, int lg_split,
                                                int vcap, unsigned int *err)
 {
-    run_item<T1>(rec, v, kNoBar, flag, G, gi, lane, xb, yb, I, O, bt, tile, lg_split, vcap, err);
+    run_item<T1>(rec, v, kNoBar, flag, G, gi, lane, xb, yb, I, O, bt, tile, lg_split, vcap, 0xffffffffu, err);
 }
 
 template <bool PDL>
@@ -271,20 +292,22 @@ plan_kernel(const BucketDev *__restrict__ buckets, int nb, int item_lo, int item
             float *yb = d.y + d.y_step * step + ((size_t)g * d.B + b0) * d.O;
             float *v = reinterpret_cast<float *>(srec + d.rec_words);
             const int vcap = (d.region_words - d.rec_words) * 4;
-            if (!staged) {
+            const uint32_t limit = (uint32_t)d.rec_words * 16u;
+            const bool t1 = d.tile == 1;
+            bool done = false;
+            if (staged)
+                done = t1 ? run_item<true>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split,
+                                           vcap, limit, &g_plan_error)
+                          : run_item<false>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, vcap,
+                                            limit, &g_plan_error);
+            if (!done) {
                 const uint4 *grec = reinterpret_cast<const uint4 *>(d.rec + (size_t)g * d.stride);
-                if (d.tile == 1)
+                if (t1)
                     run_item_in_place<true>(grec, v, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split, vcap,
                                             &g_plan_error);
                 else
                     run_item_in_place<false>(grec, v, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, vcap,
                                              &g_plan_error);
-            } else if (d.tile == 1) {
-                run_item<true>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split, vcap,
-                               &g_plan_error);
-            } else {
-                run_item<false>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, vcap,
-                                &g_plan_error);
             }
         }
         __syncthreads();
@@ -391,7 +414,8 @@ int launch_compact(neat_plan *P, int counters, cudaStream_t s)
         return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "plan: counter reset");
     }
     const int blocks = (P->n_genomes + kCompactWarps - 1) / kCompactWarps;
-    compact_kernel<<<blocks, 32 * kCompactWarps, 0, s>>>(P->d_cpops, P->n_cpops, P->n_genomes, P->d_counters, counters);
+    compact_kernel<<<blocks, 32 * kCompactWarps, 0, s>>>(P->d_cpops, P->n_cpops, CompactPop{}, P->n_genomes,
+                                                         P->d_counters, counters, nullptr);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "plan: compact launch");
 }
@@ -1248,13 +1272,26 @@ extern "C" int neat_forward_multi_noalloc(const neat_pop_desc *pops, int32_t npo
 // Internal helpers for other translation units (the serving runtime).
 namespace neat {
 
-int fill_population_bucket(const neat_pop_desc &pd, const int32_t *gidx_dev, int block_threads, int cta_begin,
-                           BucketDev *out, size_t *footprint)
+int launch_compact_population(const void *src, void *dst, int pop, const neat_dims &d, unsigned int *largest_dev,
+                              cudaStream_t s)
 {
-    const Shape sh = heuristic_shape(pd.dims.max_nodes, pd.batch, block_threads);
-    const uint32_t rec = record_max_bytes(pd.dims.num_inputs, pd.dims.num_outputs, pd.dims.max_nodes,
-                                          pd.dims.max_conns);
-    const size_t reg = ((size_t)rec + 4u * (size_t)((pd.dims.max_nodes * sh.tile + 3) & ~3) + 15) & ~(size_t)15;
+    if (pop == 0) return NEAT_OK;
+    const CompactPop one{static_cast<const uint8_t *>(src), static_cast<uint8_t *>(dst), record_stride(d), 0,
+                         d.num_inputs, d.num_outputs};
+    compact_kernel<<<(pop + kCompactWarps - 1) / kCompactWarps, 32 * kCompactWarps, 0, s>>>(nullptr, 0, one, pop, nullptr,
+                                                                                             0, largest_dev);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "compact records: launch");
+}
+
+int fill_population_bucket(const neat_pop_desc &pd, const int32_t *gidx_dev, int block_threads, int cta_begin,
+                           BucketDev *out, size_t *footprint, bool own_size, int max_used, int max_rows)
+{
+    const int rows = max_rows > 0 ? std::min(max_rows, pd.dims.max_nodes) : pd.dims.max_nodes;
+    const Shape sh = heuristic_shape(rows, pd.batch, block_threads);
+    uint32_t rec = record_max_bytes(pd.dims.num_inputs, pd.dims.num_outputs, pd.dims.max_nodes, pd.dims.max_conns);
+    if (max_used > 0) rec = std::min(rec, align16((uint32_t)max_used));
+    const size_t reg = ((size_t)rec + 4u * (size_t)((rows * sh.tile + 3) & ~3) + 15) & ~(size_t)15;
     if (!shape_ok(sh, block_threads)) return invalid("invalid launch shape for a population bucket");
     int gpc = block_threads / sh.G;
     if (sh.G > 32) gpc = std::min(gpc, 15);
@@ -1281,7 +1318,7 @@ int fill_population_bucket(const neat_pop_desc &pd, const int32_t *gidx_dev, int
     d.gpc = gpc;
     d.region_words = (int)(reg / 16);
     d.rec_words = (int)(rec / 16);
-    d.rec_copy_bytes = (int)rec;
+    d.rec_copy_bytes = own_size ? 0 : (int)rec;
     d.cta_begin = cta_begin;
     d.cta_items = (int)(((long)d.n_genomes * d.tiles + gpc - 1) / gpc);
     *footprint = reg * gpc;
