@@ -82,6 +82,27 @@ __global__ void __launch_bounds__(1024, 1) forward_kernel(const ForwardArgs a)
                  &g_forward_error);
 }
 
+// One input vector per genome, one warp per genome, the record read where it
+// lies: for records so large that staging them leaves an SM a few warps.  The
+// values alone sit in shared memory; a level's node entries and edges are
+// consecutive in memory, so a warp's reads share their lines, and the walk's
+// L2 latencies are hidden by the other warps.
+constexpr int kDirectWarps = 4;
+
+__global__ void __launch_bounds__(32 * kDirectWarps) forward_direct_kernel(const ForwardArgs a)
+{
+    extern __shared__ __align__(16) uint4 smem[];
+    __shared__ int flags[kDirectWarps];
+    const int gi = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = blockIdx.x * kDirectWarps + gi;
+    if (g >= a.pop) return;
+    float *v = reinterpret_cast<float *>(smem) + (size_t)gi * a.val_floats;
+    if (lane == 0) flags[gi] = 0;
+    run_item<true>(reinterpret_cast<const uint4 *>(a.rec + (size_t)g * a.stride), v, kNoBar, flags + gi, 32, gi, lane,
+                   a.x + (size_t)g * a.I, a.y + (size_t)g * a.O, a.I, a.O, 1, 1, 0, a.val_floats, 0xffffffffu,
+                   &g_forward_error);
+}
+
 // One thread per genome (group 1, tile 1): each thread walks the positions
 // of its own genome in order, so no barrier is needed between levels; the
 // loops run warp-uniform trip counts (the warp's largest position count and,
@@ -414,6 +435,21 @@ extern "C" int neat_forward_ex(const void *transformed_dev, int32_t pop, neat_di
     ForwardArgs a;
     int rc = make_forward_args(transformed_dev, pop, d, inputs_dev, batch, outputs_dev, L, &a);
     if (rc) return rc;
+    // no shape asked for, one vector per genome, records above 8 KB, and more
+    // genomes than two and a half waves of staged ones: at 500 / 2000 rows a
+    // staged genome takes 27 KB, eight warps an SM (4096 genomes: 27 us in
+    // place, 48 staged; 1000 / 4000: 43 and 67).  Below, the staged copy's one
+    // long read beats the walk's many short ones (300 genomes: 21 us in place,
+    // 13 staged)
+    const long staged = 152L * (long)(227u * 1024u / ((size_t)a.rec_words * 16 + (size_t)a.val_floats * 4 + 1024u));
+    if (!launch_host && batch == 1 && a.rec_copy_bytes == 0 && 2L * pop > 5L * std::max(1L, staged)) {
+        const size_t smem = 4u * (size_t)a.val_floats * kDirectWarps;
+        rc = allow_dynamic_smem(reinterpret_cast<const void *>(forward_direct_kernel), smem, "forward: shared memory per block");
+        if (rc) return rc;
+        forward_direct_kernel<<<(pop + kDirectWarps - 1) / kDirectWarps, 32 * kDirectWarps, smem, as_stream(stream)>>>(a);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "forward: launch");
+    }
     return launch_forward(a, L, as_stream(stream));
 }
 

@@ -209,6 +209,32 @@ __device__ __forceinline__ void eval_node_tile(const uint4 ne, const uint2 *__re
                                         : node_output(ne, agg, act, ec, a);
 }
 
+// walk_levels for several columns, from position `first` (the inputs before
+// it have their values); LGT: log2 of the tile's columns (-1: lgT).
+template <bool FAST, int LGT>
+__device__ __forceinline__ void walk_tile(const uint4 *nodes, const uint2 *edges, const uint16_t *lev, float *v,
+                                          int first, int n_nodes, int n_levels, int G, int gi, int lane, int lgT,
+                                          bool col_ok)
+{
+    const int lg = LGT >= 0 ? LGT : lgT;
+    const int col = lane & ((1 << lg) - 1);
+    const int sub = lane >> lg;
+    const int nsub = G >> lg;
+    if (nsub == 1) {
+        if (col_ok)
+            for (int p = first; p < n_nodes; ++p) eval_node_tile<FAST>(nodes[p], edges, v, p, lg, col);
+    } else {
+        int p0 = first;
+        for (int l = 0; l < n_levels; ++l) {
+            const int p1 = lev[l + 1];
+            if (col_ok)
+                for (int p = p0 + sub; p < p1; p += nsub) eval_node_tile<FAST>(nodes[p], edges, v, p, lg, col);
+            p0 = p1;
+            group_sync(G, gi);
+        }
+    }
+}
+
 // All non-input nodes of a staged record, for the columns this thread owns.
 //  Columns (T > 1): thread `lane` = (sub, col) computes column col of nodes
 //  sub, sub + nsub, ... of every level, nsub = G / T.
@@ -283,22 +309,11 @@ __device__ __forceinline__ void walk_levels(const uint4 *srec, float *v, int G, 
             group_sync(G, gi);
         }
     } else {
-        const int col = lane & ((1 << lgT) - 1);
-        const int sub = lane >> lgT;
-        const int nsub = G >> lgT;
-        if (nsub == 1) {
-            if (col_ok)
-                for (int p = 0; p < n_nodes; ++p) eval_node_tile<FAST>(nodes[p], edges, v, p, lgT, col);
-        } else {
-            int p0 = lev[0];
-            for (int l = 0; l < n_levels; ++l) {
-                const int p1 = lev[l + 1];
-                if (col_ok)
-                    for (int p = p0 + sub; p < p1; p += nsub) eval_node_tile<FAST>(nodes[p], edges, v, p, lgT, col);
-                p0 = p1;
-                group_sync(G, gi);
-            }
-        }
+        // 32 columns, the usual tile: a shift known at compile time makes a
+        // value's address one instruction
+        const int first = (int)(h0.w >> 16);
+        if (lgT == 5) walk_tile<FAST, 5>(nodes, edges, lev, v, first, n_nodes, n_levels, G, gi, lane, lgT, col_ok);
+        else walk_tile<FAST, -1>(nodes, edges, lev, v, first, n_nodes, n_levels, G, gi, lane, lgT, col_ok);
     }
     group_sync(G, gi);
 }

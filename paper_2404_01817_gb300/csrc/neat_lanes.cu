@@ -442,22 +442,18 @@ __global__ void __launch_bounds__(32 * kSchedWarps) lanes_sched_kernel(const uin
 }
 
 // One stable counting pass over 128 buckets by one block of 1024 threads:
-// warp k owns a contiguous range of the input order; the items in(0 .. pop-1)
-// go to put(place, item) sorted by bucket, ties in input order (the result is
-// deterministic).  An item's rank among 32 comes from a bit mask per bucket.
-template <typename In, typename BucketOf, typename Put>
-__device__ void stable_pass(int pop, In in, BucketOf bucket_of, Put put, int (*cnt)[128], uint32_t (*mask)[128],
+// warp k owns a contiguous range of the input order; out = in sorted by
+// bucket, ties in input order (the result is deterministic).
+template <typename BucketOf>
+__device__ void stable_pass(const int32_t *in, int32_t *out, int pop, BucketOf bucket_of, int (*cnt)[128],
                             int *tot)
 {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int R = (pop + 31) / 32;
     const int lo = min(pop, w * R), hi = min(pop, lo + R);
-    for (int i = threadIdx.x; i < 32 * 128; i += blockDim.x) {
-        cnt[i >> 7][i & 127] = 0;
-        mask[i >> 7][i & 127] = 0u;
-    }
+    for (int i = threadIdx.x; i < 32 * 128; i += blockDim.x) cnt[i >> 7][i & 127] = 0;
     __syncthreads();
-    for (int i = lo + lane; i < hi; i += 32) atomicAdd(&cnt[w][bucket_of(in(i))], 1);
+    for (int i = lo + lane; i < hi; i += 32) atomicAdd(&cnt[w][bucket_of(in[i])], 1);
     __syncthreads();
     if (threadIdx.x < 128) {               // per bucket total
         const int b = threadIdx.x;
@@ -494,64 +490,29 @@ __device__ void stable_pass(int pop, In in, BucketOf bucket_of, Put put, int (*c
     const unsigned below = (1u << lane) - 1u;
     for (int base = lo; base < hi; base += 32) {
         const int i = base + lane;
-        int item = 0, b = 0;
-        if (i < hi) {
-            item = in(i);
-            b = bucket_of(item);
-            atomicOr(&mask[w][b], 1u << lane);
-        }
+        const int b = i < hi ? bucket_of(in[i]) : -1 - lane;
+        const unsigned m = __match_any_sync(0xffffffffu, b);
+        if (i < hi) out[cnt[w][b] + __popc(m & below)] = in[i];
         __syncwarp();
-        const uint32_t m = i < hi ? mask[w][b] : 0u;
-        const int at = i < hi ? cnt[w][b] + __popc(m & below) : 0;
-        if (i < hi) put(at, item);
-        __syncwarp();
-        if (i < hi && lane == 31 - __clz(m)) {
-            cnt[w][b] = at + 1;
-            mask[w][b] = 0u;
-        }
+        if (i < hi && lane == 31 - __clz(m)) cnt[w][b] += __popc(m);
         __syncwarp();
     }
     __syncthreads();
 }
 
 // Genome order: most beats first, then most quads in a lane (two stable
-// passes, least significant key first).  One block: bound by the latency of
-// its passes' chains; the keys and the first pass's order stay in shared
-// memory where they fit (STAGED: two 16-bit words per genome).  10 000 genomes:
-// 17 us.
-constexpr int kSortStagedPop = 40000;
-
-template <bool STAGED>
+// passes, least significant key first).  One block.
 __global__ void __launch_bounds__(1024) lanes_sort_kernel(uint8_t *lanes, LanesGeom geo, int pop)
 {
     __shared__ int cnt[32][128];
-    __shared__ uint32_t mask[32][128];
     __shared__ int tot[128];
     const uint32_t *meas = reinterpret_cast<const uint32_t *>(lanes + geo.meas_off);
     int32_t *oa = reinterpret_cast<int32_t *>(lanes + geo.ord_a_off);
-    auto quads_key = [](uint32_t m) { return 127 - (int)min((m >> 8) & 0xffffu, 127u); };
-    auto beats_key = [](uint32_t m) { return 127 - (int)min(m & 0xffu, 127u); };
-    auto identity = [](int i) { return i; };
-    if constexpr (STAGED) {
-        uint16_t *key = reinterpret_cast<uint16_t *>(lane_sm);              // [pop] quads key | beats key << 8
-        uint16_t *first = key + pop;                                         // [pop] the first pass's order
-#pragma unroll 4
-        for (int i = threadIdx.x; i < pop; i += blockDim.x) {
-            const uint32_t m = meas[i];
-            key[i] = (uint16_t)(quads_key(m) | beats_key(m) << 8);
-        }
-        __syncthreads();
-        stable_pass(pop, identity, [&](int g) { return (int)(key[g] & 0xffu); },
-                    [&](int at, int g) { first[at] = (uint16_t)g; }, cnt, mask, tot);
-        stable_pass(pop, [&](int i) { return (int)first[i]; }, [&](int g) { return (int)(key[g] >> 8); },
-                    [&](int at, int g) { oa[at] = g; }, cnt, mask, tot);
-    } else {
-        int32_t *ob = reinterpret_cast<int32_t *>(lanes + geo.ord_b_off);
-        stable_pass(pop, identity, [&](int g) { return quads_key(meas[g]); }, [&](int at, int g) { ob[at] = g; }, cnt,
-                    mask, tot);
-        stable_pass(pop, [&](int i) { return ob[i]; }, [&](int g) { return beats_key(meas[g]); },
-                    [&](int at, int g) { oa[at] = g; }, cnt, mask, tot);
-    }
+    int32_t *ob = reinterpret_cast<int32_t *>(lanes + geo.ord_b_off);
+    for (int i = threadIdx.x; i < pop; i += blockDim.x) oa[i] = i;
+    __syncthreads();
+    stable_pass(oa, ob, pop, [&](int g) { return 127 - (int)min((meas[g] >> 8) & 0xffffu, 127u); }, cnt, tot);
+    stable_pass(ob, oa, pop, [&](int g) { return 127 - (int)min(meas[g] & 0xffu, 127u); }, cnt, tot);
 }
 
 // One warp per warp program: lane (j, k) = (lane % kLaneJ, lane / kLaneJ)
@@ -1336,15 +1297,7 @@ int lanes_pack_impl(const void *transformed_dev, int32_t pop, neat_dims d, void 
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "neat_lanes_pack: schedule");
     if (pop == 0) return NEAT_OK;
-    if (pop <= kSortStagedPop) {
-        const size_t sort_smem = 4u * (size_t)pop;
-        rc = allow_dynamic_smem(reinterpret_cast<const void *>(lanes_sort_kernel<true>), sort_smem,
-                                "neat_lanes_pack: shared memory");
-        if (rc) return rc;
-        lanes_sort_kernel<true><<<1, 1024, sort_smem, s>>>(L, g, pop);
-    } else {
-        lanes_sort_kernel<false><<<1, 1024, 0, s>>>(L, g, pop);
-    }
+    lanes_sort_kernel<<<1, 1024, 0, s>>>(L, g, pop);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "neat_lanes_pack: sort");
     lanes_pack_kernel<<<g.warps, 32, pack_smem, s>>>(rec, stride, pop, d.num_inputs, d.num_outputs, N, g.rec_bytes, L,
