@@ -30,7 +30,8 @@ __device__ unsigned int g_forward_error;
 
 // One work item per group of a.group threads.  T1: one input vector per
 // genome (tile 1), the case of a control loop that steps every genome once.
-template <bool PDL, bool T1>
+// PAIRS: two columns per thread.
+template <bool PDL, bool T1, bool PAIRS = false>
 __global__ void __launch_bounds__(1024, 1) forward_kernel(const ForwardArgs a)
 {
     extern __shared__ __align__(16) uint4 smem[];
@@ -77,9 +78,9 @@ __global__ void __launch_bounds__(1024, 1) forward_kernel(const ForwardArgs a)
         pdl_wait();
         pdl_trigger();
     }
-    run_item<T1>(srec, v, bar, flags + gi, G, gi, lane, a.x + ((size_t)g * a.B + b0) * a.I,
-                 a.y + ((size_t)g * a.B + b0) * a.O, a.I, a.O, bt, a.tile, a.lg_split, a.val_floats, 0xffffffffu,
-                 &g_forward_error);
+    run_item<T1, PAIRS>(srec, v, bar, flags + gi, G, gi, lane, a.x + ((size_t)g * a.B + b0) * a.I,
+                        a.y + ((size_t)g * a.B + b0) * a.O, a.I, a.O, bt, a.tile, a.lg_split, a.val_floats, 0xffffffffu,
+                        &g_forward_error);
 }
 
 // One input vector per genome, one warp per genome, the record read where it
@@ -266,6 +267,7 @@ int make_forward_args(const void *transformed, int32_t pop, const neat_dims &d, 
     a.val_floats = (a.N * L.tile + 3) & ~3;
     a.rec_copy_bytes = (a.rec_words * 16 <= kOnePieceRecordBytes) ? a.rec_words * 16 : 0;
     a.order = L.order_dev;
+    a.pairs = 0;
     *out = a;
     return NEAT_OK;
 }
@@ -277,7 +279,7 @@ int launch_forward(const ForwardArgs &a, const neat_launch &L, cudaStream_t s)
     const size_t per_group = (size_t)a.rec_words * 16 + (size_t)a.val_floats * 4;
     const size_t smem = per_group * L.groups_per_block + 16u * (size_t)forward_header_words(L.groups_per_block);
     if (smem > 227 * 1024) return invalid("forward: shared memory per block exceeds 227 KB; lower tile or groups_per_block");
-    KernelFn f = pick(L.pdl != 0, a.tile == 1);
+    KernelFn f = a.pairs ? forward_kernel<false, false, true> : pick(L.pdl != 0, a.tile == 1);
     if (L.group == 1 && a.tile == 1) {
         // one thread per genome; the whole record is copied in one piece
         if (a.rec_copy_bytes == 0) return invalid("forward: group 1 needs records of at most 8 KB");
@@ -449,6 +451,26 @@ extern "C" int neat_forward_ex(const void *transformed_dev, int32_t pop, neat_di
         forward_direct_kernel<<<(pop + kDirectWarps - 1) / kDirectWarps, 32 * kDirectWarps, smem, as_stream(stream)>>>(a);
         const cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "forward: launch");
+    }
+    if (!launch_host && batch > 32) {
+        // two columns per thread in tiles of 64, where four such groups fit an
+        // SM.  1001 genomes of 101 / 403 rows and 37 vectors: 51 -> 46 us with
+        // the transform (one tile of 37 instead of tiles of 32 and 5).  (In the
+        // plan's kernel, whose registers it overran, the same shapes took 195
+        // instead of 189 us a step)
+        neat_launch W = L;
+        W.tile = 64;
+        W.group = 32 * tile_row_threads(d.max_nodes);
+        const size_t per_group = (size_t)a.rec_words * 16 + 4u * 64u * (size_t)d.max_nodes;
+        if (per_group <= kMaxPairGroupSmem) {
+            a.pairs = 1;
+            a.tile = W.tile;
+            a.group = W.group;
+            a.tiles = (batch + W.tile - 1) / W.tile;
+            a.val_floats = a.N * W.tile;
+            W.groups_per_block = groups_per_block_for((long)pop * a.tiles, W.group, per_group);
+            return launch_forward(a, W, as_stream(stream));
+        }
     }
     return launch_forward(a, L, as_stream(stream));
 }

@@ -57,6 +57,9 @@ int allow_dynamic_smem(const void *kernel, size_t dynamic_bytes, const char *wha
 // Shared memory one group's record and value tiles may take in a default
 // launch shape (room left for the block's barriers).
 constexpr size_t kMaxGroupSmem = 200u * 1024u;
+// The same for a tile of 64 columns, two per thread: beyond, fewer than four
+// groups share an SM and the tile of 32 is the better one.
+constexpr size_t kMaxPairGroupSmem = 48u * 1024u;
 
 // Threads per tile row for a genome of up to n nodes and a batch of several
 // input vectors: about one per 32 nodes (a level of a large genome holds
@@ -83,6 +86,7 @@ struct ForwardArgs {
     int val_floats;          // floats of shared memory for node values (N * tile, rounded to 4)
     int rec_copy_bytes;      // bytes of each record copied in one piece (0: read the size from its header)
     const int32_t *order;    // genome of work item k / tiles (NULL: identity)
+    int pairs;               // two columns per thread (tile at most 2 x group)
 };
 
 // 16-byte words before the groups' regions in a forward block's shared

@@ -235,6 +235,143 @@ __device__ __forceinline__ void walk_tile(const uint4 *nodes, const uint2 *edges
     }
 }
 
+// ---- two adjacent columns per thread
+//
+// A row of T columns is evaluated by T / 2 threads, columns 2 l and 2 l + 1 in
+// thread l: the node's entry, its dispatches and its edges are read once for
+// both, their values are one 8-byte read and their sums run as a packed pair.
+// Each column's operations are those of eval_node_tile in the same order, so
+// the bits are too.
+template <int EC>
+__device__ __forceinline__ f2 sum_edges_pair(const uint2 *__restrict__ e, const char *__restrict__ v, int lgT)
+{
+    f2 q[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+    for (int i = 0; i < EC; ++i) {
+        const uint2 t = e[i];
+        const f2 x = *reinterpret_cast<const f2 *>(v + ((size_t)t.y << (lgT + 2)));
+        q[i & 3] = fma2(pack2(__uint_as_float(t.x), __uint_as_float(t.x)), x, q[i & 3]);
+    }
+    return add2(add2(q[0], q[1]), add2(q[2], q[3]));
+}
+
+__device__ __forceinline__ f2 sum_edges_pair_any(const uint2 *__restrict__ e, uint32_t ec, const char *__restrict__ v,
+                                                 int lgT)
+{
+    f2 q[4] = {0ull, 0ull, 0ull, 0ull};
+    for (uint32_t i = 0; i < ec; i += 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k < ec) {
+                const uint2 t = e[i + k];
+                const f2 x = *reinterpret_cast<const f2 *>(v + ((size_t)t.y << (lgT + 2)));
+                q[k] = fma2(pack2(__uint_as_float(t.x), __uint_as_float(t.x)), x, q[k]);
+            }
+        }
+    }
+    return add2(add2(q[0], q[1]), add2(q[2], q[3]));
+}
+
+template <uint32_t AGG>
+__device__ __forceinline__ float2 fold_edges_pair(const uint2 *__restrict__ e, uint32_t ec, const char *__restrict__ v,
+                                                  int lgT)
+{
+    float q[4][2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) q[k][0] = q[k][1] = agg_identity(AGG);
+    for (uint32_t i = 0; i < ec; i += 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k < ec) {
+                const uint2 t = e[i + k];
+                const float2 x = *reinterpret_cast<const float2 *>(v + ((size_t)t.y << (lgT + 2)));
+                q[k][0] = agg_step(AGG, q[k][0], __uint_as_float(t.x), x.x);
+                q[k][1] = agg_step(AGG, q[k][1], __uint_as_float(t.x), x.y);
+            }
+        }
+    }
+    return make_float2(agg_combine(AGG, agg_combine(AGG, q[0][0], q[1][0]), agg_combine(AGG, q[2][0], q[3][0])),
+                       agg_combine(AGG, agg_combine(AGG, q[0][1], q[1][1]), agg_combine(AGG, q[2][1], q[3][1])));
+}
+
+// Node p for the thread's columns; v: the thread's place in row 0.
+template <bool FAST>
+__device__ __forceinline__ void eval_node_pair(const uint4 ne, const uint2 *__restrict__ edges, char *__restrict__ v,
+                                               int p, int lgT)
+{
+    const uint32_t act = ne.w & 0xffu;
+    if (act == kInputAct) return;
+    const uint32_t agg = FAST ? kAggSum : ((ne.w >> 8) & 0xffu);
+    const uint32_t ec = ne.z >> 16;
+    const uint2 *e = edges + (ne.z & 0xffffu);
+    float2 a;
+    if (FAST || agg == kAggSum || agg == kAggMean) {
+        f2 s;
+        switch (ec) {
+        case 0: s = 0ull; break;
+        case 1: s = sum_edges_pair<1>(e, v, lgT); break;
+        case 2: s = sum_edges_pair<2>(e, v, lgT); break;
+        case 3: s = sum_edges_pair<3>(e, v, lgT); break;
+        case 4: s = sum_edges_pair<4>(e, v, lgT); break;
+        case 5: s = sum_edges_pair<5>(e, v, lgT); break;
+        case 6: s = sum_edges_pair<6>(e, v, lgT); break;
+        default: s = sum_edges_pair_any(e, ec, v, lgT);
+        }
+        a = unpack2(s);
+        if (!FAST && agg == kAggMean && ec > 0) {
+            a.x = a.x / (float)ec;
+            a.y = a.y / (float)ec;
+        }
+    } else {
+        a = agg == kAggProduct ? fold_edges_pair<kAggProduct>(e, ec, v, lgT) : fold_edges_pair<kAggMax>(e, ec, v, lgT);
+        if (ec == 0) a = make_float2(0.0f, 0.0f);
+    }
+    const float r = __uint_as_float(ne.y), b = __uint_as_float(ne.x);
+    const float z0 = fmaf(r, a.x, b), z1 = fmaf(r, a.y, b);
+    float2 y;
+    if (FAST) {
+        y = make_float2(node_tanh(z0), node_tanh(z1));
+    } else {
+        switch (act) {                            // one dispatch for both
+        case 1: y = make_float2(activate(1, z0), activate(1, z1)); break;
+        case 2: y = make_float2(activate(2, z0), activate(2, z1)); break;
+        case 3: y = make_float2(activate(3, z0), activate(3, z1)); break;
+        case 4: y = make_float2(activate(4, z0), activate(4, z1)); break;
+        case 5: y = make_float2(activate(5, z0), activate(5, z1)); break;
+        case 6: y = make_float2(activate(6, z0), activate(6, z1)); break;
+        default: y = make_float2(z0, z1);
+        }
+    }
+    *reinterpret_cast<float2 *>(v + ((size_t)p << (lgT + 2))) = y;
+}
+
+// walk_levels for two columns per thread: 2^lgT columns (at least 2), of which
+// the first `cols` are asked for.
+template <bool FAST>
+__device__ __forceinline__ void walk_pairs(const uint4 *srec, float *v, int G, int gi, int lane, int lgT, int cols)
+{
+    const uint4 h0 = srec[0], h1 = srec[1];
+    const int n_levels = (int)(h0.x >> 16);
+    const uint4 *nodes = srec + 2;
+    const uint2 *edges = reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(srec) + h1.y);
+    const uint16_t *lev = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.z);
+    const int pair = lane & ((1 << (lgT - 1)) - 1), sub = lane >> (lgT - 1), nsub = G >> (lgT - 1);
+    char *mine = reinterpret_cast<char *>(v + 2 * pair);
+    const bool ok = 2 * pair < cols;
+    int p0 = (int)(h0.w >> 16);
+    for (int l = 0; l < n_levels; ++l) {
+        const int p1 = lev[l + 1];
+        if (ok)
+            for (int p = p0 + sub; p < p1; p += nsub) {
+                if (lgT == 6) eval_node_pair<FAST>(nodes[p], edges, mine, p, 6);
+                else eval_node_pair<FAST>(nodes[p], edges, mine, p, lgT);
+            }
+        p0 = p1;
+        if (nsub > 1) group_sync(G, gi);
+    }
+    group_sync(G, gi);
+}
+
 // All non-input nodes of a staged record, for the columns this thread owns.
 //  Columns (T > 1): thread `lane` = (sub, col) computes column col of nodes
 //  sub, sub + nsub, ... of every level, nsub = G / T.
@@ -337,8 +474,9 @@ constexpr uint32_t kNoBar = 0xffffffffu;
 //   the value tile, at least one column of the genome's nodes (a genome with
 //   more nodes than the tile has rows takes fewer columns at a time).
 // False, with nothing evaluated, when the record is longer than rec_limit
-// bytes (the part that was copied).
-template <bool T1>
+// bytes (the part that was copied).  PAIRS: two columns per thread (tile at
+// least 2, at most 2 G; vcap at least two columns).
+template <bool T1, bool PAIRS = false>
 __device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t bar, volatile int *flag, int G,
                                          int gi, int lane, const float *__restrict__ xb, float *__restrict__ yb,
                                          int I, int O, int bt, int tile, int lg_split, int vcap, uint32_t rec_limit,
@@ -369,7 +507,7 @@ __device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t b
     if (h1.x > rec_limit) return false;
     const uint16_t *io = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.w);
     if constexpr (!T1)
-        while (lgT > 0 && ((int)(h0.x & 0xffffu) << lgT) > vcap) --lgT;
+        while (lgT > (PAIRS ? 1 : 0) && ((int)(h0.x & 0xffffu) << lgT) > vcap) --lgT;
     const int step = T1 ? 1 : 1 << lgT;
     for (int c0 = 0; c0 < bt; c0 += step) {                 // once, unless the nodes outgrow the tile's rows
         const int cols = T1 ? 1 : min(bt - c0, step);
@@ -402,7 +540,11 @@ __device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t b
         }
         group_sync(G, gi);
         const bool col_ok = T1 || (lane & (step - 1)) < cols;
-        if ((h0.w & 0xffffu) == kTraitsSumTanh) walk_levels<T1, true>(srec, v, G, gi, lane, lgT, lg_split, col_ok);
+        const bool fast = (h0.w & 0xffffu) == kTraitsSumTanh;
+        if constexpr (PAIRS) {
+            if (fast) walk_pairs<true>(srec, v, G, gi, lane, lgT, cols);
+            else walk_pairs<false>(srec, v, G, gi, lane, lgT, cols);
+        } else if (fast) walk_levels<T1, true>(srec, v, G, gi, lane, lgT, lg_split, col_ok);
         else walk_levels<T1, false>(srec, v, G, gi, lane, lgT, lg_split, col_ok);
         for (int i = lane; i < cols * O; i += G) {
             if (T1) yb[i] = v[io[I + i]];
