@@ -195,7 +195,10 @@ NEAT_API int neat_transform(const float *nodes_dev, const float *conns_dev, int3
  *   transformed_dev  records written by neat_transform with the same dims
  *   inputs_dev       f32 [pop][batch][I]
  *   outputs_dev      f32 [pop][batch][O] (written; NaN for genomes with an error bit)
- * The launch shape is chosen from (dims, batch); the results do not depend on it.
+ * The launch shape is chosen from (pop, dims, batch), as neat_default_launch
+ * says; batches above 32 are evaluated two input vectors per thread where the
+ * genomes' values are small enough, and one vector for many large genomes reads
+ * the records where they lie.  The results do not depend on it.
  * Errors: NEAT_EINVAL, NEAT_ECUDA.
  */
 NEAT_API int neat_forward(const void *transformed_dev, int32_t pop, neat_dims d,
@@ -235,8 +238,8 @@ typedef struct neat_launch {
  */
 NEAT_API int neat_schedule(const void *transformed_dev, int32_t pop, neat_dims d, int32_t *order_dev, void *stream);
 
-/* The launch shape neat_forward uses for (pop, d, batch): for one input
- * vector per genome, 8 to 32 threads per genome by max_nodes; for several,
+/* The staged launch shape for (pop, d, batch), which neat_forward uses but for
+ * the two forms it names: for one input vector per genome, 8 to 32 threads per genome by max_nodes; for several,
  * tiles of up to 32 vectors with a power of two of threads per tile row
  * (about one per 32 nodes, at most 16), the tile halved until a group's
  * record and value tile fit one block; then the number of groups per block
@@ -295,7 +298,8 @@ NEAT_API int neat_forward_fused(const void *transformed_dev, int32_t pop, neat_d
  * neat_lanes_info.unordered).
  *
  * Compilation: per genome a list schedule of beats of up to two nodes whose
- * sources are all computed in earlier beats (longest remaining path first);
+ * sources are all computed in earlier beats (longest remaining path first),
+ * without the nodes that no output depends on;
  * genomes sorted by (beats, edge quads), deepest first, 16 to a warp; each
  * warp program holds its beats' node entries and the nodes' incoming edges
  * in quads of four, interleaved by lane.
@@ -597,7 +601,9 @@ NEAT_API int neat_fill_words(uint64_t seed, uint64_t stream, uint32_t *words_dev
  * `layers` layers, each a res x res grid over [-1,1]^2 with coordinate
  * -1 + 2 i / (res - 1) (computed in double, rounded to float) and node index
  * res * iy + ix.  The weight is the CPPN output, set to 0 when
- * |w| < threshold (the comparison made in float32).
+ * |w| < threshold (the comparison made in float32).  The layers share one grid
+ * and a query holds no layer coordinate, so every block has the same weight at
+ * the same (source, target): each pair is evaluated once.
  */
 typedef struct neat_substrate {
     int32_t resolution;   /* nodes per side of a layer, 2..181 */
@@ -641,6 +647,12 @@ NEAT_API int neat_substrate_forward(const float *weights_dev, int32_t pop, neat_
  * blocks pull work from a device counter, so uneven buckets balance across
  * SMs.  Results are bit-identical to neat_forward on each population (the
  * aggregation order is a function of the genome alone).
+ * Where it saves more than it costs, every call first copies the records to
+ * compact ones (a workspace of the records' size, held by the plan) without
+ * the nodes that no output depends on; buckets and shapes then follow the
+ * compact records.  The copy is made from the records as they are at the call:
+ * records may be written anew between calls (any genomes of the same dims), and
+ * ones that outgrow the plan's shapes are evaluated all the same, slower.
  */
 typedef struct neat_pop_desc {
     const void *transformed_dev;   /* records from neat_transform */
@@ -670,8 +682,8 @@ typedef struct neat_plan neat_plan;
 NEAT_API int neat_plan_create(const neat_pop_desc *pops_host, int32_t npops, const neat_plan_options *opt_host,
                               void *stream, neat_plan **out_host);
 
-/* One step for every population of the plan (one kernel launch, plus a
- * counter reset). */
+/* One step for every population of the plan (one kernel launch, after the
+ * compact copy or a counter reset). */
 NEAT_API int neat_plan_forward(neat_plan *plan, int32_t step, void *stream);
 
 /* Steps first_step .. first_step+steps-1 as one CUDA graph (built on first
@@ -717,7 +729,9 @@ NEAT_API int neat_forward_multi_noalloc(const neat_pop_desc *pops_host, int32_t 
  * pool of hbm_budget_bytes (allocated at create) and a scheduler thread.
  * Queued requests are admitted, in arrival order (a later one that fits may
  * pass one that does not), as pool memory frees up; their genome tensors are
- * copied in and transformed once.  Every scheduler tick advances each active
+ * copied in and transformed once, then copied without the nodes that no output
+ * depends on into the memory of the genome tensors, where that is large enough.
+ * Every scheduler tick advances each active
  * request by one step -- one kernel generating the step's observations, one
  * persistent-kernel launch evaluating all active requests together -- so
  * requests that arrive while others run share the device with them.  A

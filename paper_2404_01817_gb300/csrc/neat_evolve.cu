@@ -19,11 +19,12 @@
 // (in, out) pairs in shared-memory hash tables (lowest row per key or pair)
 // looked up for every row of the first parent.
 //
-// The warp forms are bound by memory latency (long-scoreboard stalls at 40 to
-// 45% of the warps, 34 to 45% of the issue slots).  10 000 Ant-sized genomes:
-// mutation 44 us (block of 64 threads per genome: 80 us, 3490 against 1510
-// warp instructions per genome), crossover 38 us (block of 128: 75 us, 4900
-// against 1710).
+// The warp forms are bound by memory latency (long-scoreboard stalls at 36 to
+// 45% of the warps, 45 to 47% of the issue slots).  10 000 Ant-sized genomes:
+// mutation 34 us (block of 64 threads per genome: 80 us, 3490 against 1520
+// warp instructions per genome; with loops whose remainders wait for each row
+// 44 us), crossover 38 us (block of 128: 75 us, 4900 against 1710; with its
+// lookups' rows loaded together, which takes 64 registers, no faster).
 #include <algorithm>
 
 #include "neat_device.cuh"
@@ -140,6 +141,7 @@ __device__ int select_choose(int R, Pred pred, uint32_t u, int *s_cnt, int *s_ro
 // check a sweep over predecessor masks.
 constexpr int kWarpNodes = 128, kWarpConns = 512;
 constexpr unsigned kAll = 0xffffffffu;
+constexpr int kBatch = 4;                // rows a lane has in flight at once
 
 // The mask of rows 32k .. 32k+31 of [0, R) that satisfy pred, on lane k.
 template <typename Pred>
@@ -215,10 +217,26 @@ __global__ void __launch_bounds__(128) mutate_warp_kernel(const MutArgs a)
     const float *z = a.normals + (size_t)g * a.Z;
 
     const uint32_t word = lane < 9 ? __ldg(u + lane) : 0u;        // the structural words
-#pragma unroll 4
-    for (int c = lane; c < C; c += 32) cs[c] = conns[c];
-#pragma unroll 4
-    for (int i = lane; i < 5 * N; i += 32) ns[i] = nodes[i];
+    // loads in whole batches, past the last row too (predicated off): a loop's
+    // remainder would wait for every row by itself
+    for (int base = lane; base < C; base += 32 * kBatch) {
+        float4 row[kBatch];
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j)
+            if (base + 32 * j < C) row[j] = conns[base + 32 * j];
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j)
+            if (base + 32 * j < C) cs[base + 32 * j] = row[j];
+    }
+    for (int base = lane; base < 5 * N; base += 64 * kBatch) {
+        float x[2 * kBatch];
+#pragma unroll
+        for (int j = 0; j < 2 * kBatch; ++j)
+            if (base + 32 * j < 5 * N) x[j] = nodes[base + 32 * j];
+#pragma unroll
+        for (int j = 0; j < 2 * kBatch; ++j)
+            if (base + 32 * j < 5 * N) ns[base + 32 * j] = x[j];
+    }
     __syncwarp();
     auto u_at = [&](int k) { return __shfl_sync(kAll, word, k); };
     auto node_present = [&](int r) { return !isnan(ns[5 * r]); };
@@ -358,38 +376,77 @@ __global__ void __launch_bounds__(128) mutate_warp_kernel(const MutArgs a)
     const float in_end = (float)a.I;
     const uint32_t *wc = u + kStructWords + 6 * (size_t)N;
     const float *zc = z + kStructNormals + 2 * (size_t)N;
-#pragma unroll 4
-    for (int c = lane; c < C; c += 32) {
-        float4 x = cs[c];
-        const uint32_t w0 = __ldg(wc + 2 * (size_t)c);
-        const uint32_t w1 = a.t_en ? __ldg(wc + 2 * (size_t)c + 1) : 0xffffffffu;
-        const float zz = __ldg(zc + c);
-        if (!(isnan(x.x) || isnan(x.y) || isnan(x.z))) {
-            if (below(w0, a.t_w_m)) x.w = fmaf(a.w_power, zz, x.w);
-            else if (below(w0, a.t_w_mr)) x.w = fmaf(a.w_std, zz, a.w_mean);
-            if (a.t_en && below(w1, a.t_en)) x.z = (x.z != 0.0f) ? 0.0f : 1.0f;
+    for (int base = lane; base < C; base += 32 * kBatch) {
+        uint32_t w0[kBatch], w1[kBatch];
+        float zz[kBatch];
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const int c = base + 32 * j;
+            w0[j] = w1[j] = 0xffffffffu;
+            zz[j] = 0.0f;
+            if (c < C) {
+                w0[j] = __ldg(wc + 2 * (size_t)c);
+                if (a.t_en) w1[j] = __ldg(wc + 2 * (size_t)c + 1);
+                zz[j] = __ldg(zc + c);
+            }
         }
-        conns[c] = x;
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const int c = base + 32 * j;
+            if (c >= C) break;
+            float4 x = cs[c];
+            if (!(isnan(x.x) || isnan(x.y) || isnan(x.z))) {
+                if (below(w0[j], a.t_w_m)) x.w = fmaf(a.w_power, zz[j], x.w);
+                else if (below(w0[j], a.t_w_mr)) x.w = fmaf(a.w_std, zz[j], a.w_mean);
+                if (a.t_en && below(w1[j], a.t_en)) x.z = (x.z != 0.0f) ? 0.0f : 1.0f;
+            }
+            conns[c] = x;
+        }
     }
-    for (int r = lane; r < N; r += 32) {
-        float *n = ns + 5 * r;
-        if (isnan(n[0]) || n[0] < in_end) continue;
-        const uint32_t *w = u + kStructWords + 6 * (size_t)r;
-        const float *zz = z + kStructNormals + 2 * (size_t)r;
-        if (a.t_bias_m | a.t_bias_mr) {
-            const uint32_t w0 = __ldg(w);
-            const float z0 = __ldg(zz);
-            if (below(w0, a.t_bias_m)) n[1] = fmaf(a.bias_power, z0, n[1]);
-            else if (below(w0, a.t_bias_mr)) n[1] = fmaf(a.bias_std, z0, a.bias_mean);
+    for (int base = lane; base < N; base += 64) {
+        // two rows a lane; only the words that some rate can use
+        uint32_t wr[2][6];
+        float zr[2][2];
+        bool on[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int r = base + 32 * j;
+            on[j] = r < N && !isnan(ns[5 * min(r, N - 1)]) && ns[5 * min(r, N - 1)] >= in_end;
+            const uint32_t *w = u + kStructWords + 6 * (size_t)r;
+            const float *zz = z + kStructNormals + 2 * (size_t)r;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) wr[j][k] = 0xffffffffu;
+            zr[j][0] = zr[j][1] = 0.0f;
+            if (on[j]) {
+                if (a.t_bias_m | a.t_bias_mr) {
+                    wr[j][0] = __ldg(w);
+                    zr[j][0] = __ldg(zz);
+                }
+                if (a.t_resp_m | a.t_resp_mr) {
+                    wr[j][1] = __ldg(w + 1);
+                    zr[j][1] = __ldg(zz + 1);
+                }
+                if (a.t_act && a.n_act > 0) {
+                    wr[j][2] = __ldg(w + 2);
+                    wr[j][3] = __ldg(w + 3);
+                }
+                if (a.t_agg && a.n_agg > 0) {
+                    wr[j][4] = __ldg(w + 4);
+                    wr[j][5] = __ldg(w + 5);
+                }
+            }
         }
-        if (a.t_resp_m | a.t_resp_mr) {
-            const uint32_t w1 = __ldg(w + 1);
-            const float z1 = __ldg(zz + 1);
-            if (below(w1, a.t_resp_m)) n[2] = fmaf(a.resp_power, z1, n[2]);
-            else if (below(w1, a.t_resp_mr)) n[2] = fmaf(a.resp_std, z1, a.resp_mean);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            if (!on[j]) continue;
+            float *n = ns + 5 * (base + 32 * j);
+            if (below(wr[j][0], a.t_bias_m)) n[1] = fmaf(a.bias_power, zr[j][0], n[1]);
+            else if (below(wr[j][0], a.t_bias_mr)) n[1] = fmaf(a.bias_std, zr[j][0], a.bias_mean);
+            if (below(wr[j][1], a.t_resp_m)) n[2] = fmaf(a.resp_power, zr[j][1], n[2]);
+            else if (below(wr[j][1], a.t_resp_mr)) n[2] = fmaf(a.resp_std, zr[j][1], a.resp_mean);
+            if (a.t_act && a.n_act > 0 && below(wr[j][2], a.t_act)) n[4] = (float)a.act_opt[choose(wr[j][3], a.n_act)];
+            if (a.t_agg && a.n_agg > 0 && below(wr[j][4], a.t_agg)) n[3] = (float)a.agg_opt[choose(wr[j][5], a.n_agg)];
         }
-        if (a.t_act && a.n_act > 0 && below(__ldg(w + 2), a.t_act)) n[4] = (float)a.act_opt[choose(__ldg(w + 3), a.n_act)];
-        if (a.t_agg && a.n_agg > 0 && below(__ldg(w + 4), a.t_agg)) n[3] = (float)a.agg_opt[choose(__ldg(w + 5), a.n_agg)];
     }
     __syncwarp();
 #pragma unroll 4
