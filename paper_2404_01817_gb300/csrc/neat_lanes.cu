@@ -699,8 +699,8 @@ __device__ __forceinline__ void store_value(char *V, uint32_t dst, int lane, flo
 // tiles and writes the other); SYNC: a warp barrier after every beat (the
 // feedforward walk reads values written in earlier beats; the recurrent
 // walk reads only the previous iteration's tile).
-template <bool FAST, uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true>
-__device__ __forceinline__ void walk(const unsigned char *__restrict__ P, int nb, float *V, int lane)
+template <bool FAST, uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true, int W = 1>
+__device__ __forceinline__ void walk(const unsigned char *__restrict__ P, int nb, float *V, int lane, int warp = 0)
 {
     const uint32_t off_node = kWarpSbOff + align16(4u * (uint32_t)nb);
     const uint32_t *sbt = reinterpret_cast<const uint32_t *>(P + kWarpSbOff);
@@ -708,7 +708,7 @@ __device__ __forceinline__ void walk(const unsigned char *__restrict__ P, int nb
     const unsigned char *R = P + off_node + 512u * (uint32_t)nb + 24u * (uint32_t)lane;
     const char *Vc = reinterpret_cast<const char *>(V);
     char *Vw = reinterpret_cast<char *>(V);
-    for (int b = 0; b < nb; ++b) {
+    for (int b = warp; b < nb; b += W) {
         const int T = (int)(sbt[b] & 0xffffu);
         const uint4 ne = nodes[32 * b];
         const uint32_t ec = ne.w & 0xffffu;
@@ -814,18 +814,18 @@ __device__ __forceinline__ void load_beat_head(BeatState &st, uint4 ne, uint32_t
     for (int t = 0; t < kHeadRows; ++t) st.q[t] = lds_quad((uint32_t)t < st.mt ? st.base + (uint32_t)t * kRowBytes : ra);
 }
 
-// `len` beats from beat b on, every one with T trips (T even, known at
+// The warp's beats from b up to `end`, every one with T trips (T even, known at
 // compile time; T = 0: nodes without edges).  Per beat: rows kHeadRows..T-1
 // loaded (the first rows are in the state), then the values and the fused
 // multiply-adds in trip order per partial; the next beat's head (entry and
 // first rows) is loaded before the node rule, the store of the value into
 // every column of the genome and the warp barrier.  A lane past its own
 // quads reads the padding quad at `ra`.
-template <int T, uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true>
-__device__ __forceinline__ void run_beats(BeatState &st, int b, int len, int nb, uint32_t na, uint32_t ra, int lane)
+template <int T, uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true, int W = 1>
+__device__ __forceinline__ void run_beats(BeatState &st, int &b, int end, int nb, uint32_t na, uint32_t ra, int lane)
 {
-    for (int i = 0; i < len; ++i, ++b) {
-        const uint4 nn = b + 1 < nb ? lds_u4(na + 512u * (uint32_t)(b + 1)) : st.ne;
+    for (; b < end; b += W) {
+        const uint4 nn = b + W < nb ? lds_u4(na + 512u * (uint32_t)(b + W)) : st.ne;
         float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;
         if (T > 0) {
             Quad q[T > 0 ? T : 1];
@@ -848,12 +848,12 @@ __device__ __forceinline__ void run_beats(BeatState &st, int b, int len, int nb,
 }
 
 // The same for any even T above 8 (trip pairs in a loop after the head rows).
-template <uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true>
-__device__ __forceinline__ void run_beats_any(BeatState &st, int T, int b, int len, int nb, uint32_t na, uint32_t ra,
-                                           int lane)
+template <uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true, int W = 1>
+__device__ __forceinline__ void run_beats_any(BeatState &st, int T, int &b, int end, int nb, uint32_t na, uint32_t ra,
+                                              int lane)
 {
-    for (int i = 0; i < len; ++i, ++b) {
-        const uint4 nn = b + 1 < nb ? lds_u4(na + 512u * (uint32_t)(b + 1)) : st.ne;
+    for (; b < end; b += W) {
+        const uint4 nn = b + W < nb ? lds_u4(na + 512u * (uint32_t)(b + W)) : st.ne;
         float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;
 #pragma unroll
         for (int t = 0; t < kHeadRows; ++t)
@@ -880,28 +880,32 @@ __device__ __forceinline__ void run_beats_any(BeatState &st, int T, int b, int l
 // per run to a loop compiled for that count (one code path per loop keeps
 // the hot loop compact; dispatching per beat measured ~120 cycles slower
 // per beat).
-template <uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true>
-__device__ __forceinline__ void walk_fast_staged(uint32_t P, int nb, int lane)
+// W warps share the beats of a recurrent program, which do not depend on one
+// another: warp w takes beats w, w + W, ...
+template <uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true, int W = 1>
+__device__ __forceinline__ void walk_fast_staged(uint32_t P, int nb, int lane, int warp = 0)
 {
     const uint32_t off_node = kWarpSbOff + align16(4u * (uint32_t)nb);
     const uint32_t sa = P + kWarpSbOff;
     const uint32_t na = P + off_node + 16u * (uint32_t)lane;
     const uint32_t ra = P + off_node + 512u * (uint32_t)nb + 24u * (uint32_t)lane;   // row 0: padding quad
-    if (nb <= 0) return;
+    if (warp >= nb) return;
     BeatState st;
-    load_beat_head(st, lds_u4(na), ra);
-    for (int b = 0; b < nb;) {
-        const uint32_t e = lds_u32(sa + 4u * (uint32_t)b);
-        const int T = (int)(e & 0xffffu), len = max(1, (int)(e >> 16));
+    load_beat_head(st, lds_u4(na + 512u * (uint32_t)warp), ra);
+    int b = warp;                                     // the warp's next beat
+    for (int run = 0; run < nb;) {
+        const uint32_t e = lds_u32(sa + 4u * (uint32_t)run);
+        const int T = (int)(e & 0xffffu);
+        run += max(1, (int)(e >> 16));
+        const int end = min(run, nb);
         switch (T) {
-        case 0: run_beats<0, RD, WR, SYNC>(st, b, len, nb, na, ra, lane); break;
-        case 2: run_beats<2, RD, WR, SYNC>(st, b, len, nb, na, ra, lane); break;
-        case 4: run_beats<4, RD, WR, SYNC>(st, b, len, nb, na, ra, lane); break;
-        case 6: run_beats<6, RD, WR, SYNC>(st, b, len, nb, na, ra, lane); break;
-        case 8: run_beats<8, RD, WR, SYNC>(st, b, len, nb, na, ra, lane); break;
-        default: run_beats_any<RD, WR, SYNC>(st, T, b, len, nb, na, ra, lane);
+        case 0: run_beats<0, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
+        case 2: run_beats<2, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
+        case 4: run_beats<4, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
+        case 6: run_beats<6, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
+        case 8: run_beats<8, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
+        default: run_beats_any<RD, WR, SYNC, W>(st, T, b, end, nb, na, ra, lane);
         }
-        b += len;
     }
 }
 
@@ -1054,19 +1058,22 @@ __global__ void __launch_bounds__(32) lanes_kernel(const LanesArgs a)
 __host__ __device__ inline uint32_t lanes_rnn_tile_bytes(int N) { return (uint32_t)(N + 3) * 256u; }
 
 // One iteration of a recurrent warp program: every beat reads tile RD and
-// writes tile WR (byte offsets 0 / 128), no barrier between beats.
-template <uint32_t RD, uint32_t WR>
+// writes tile WR (byte offsets 0 / 128), so that beats need no barrier and no
+// order among them; the block's W warps take turns.
+template <uint32_t RD, uint32_t WR, int W>
 __device__ __forceinline__ void rnn_iteration(const unsigned char *sprog, const unsigned char *gw, bool staged,
-                                              bool fast, int nb, float *V, int lane)
+                                              bool fast, int nb, float *V, int lane, int warp)
 {
     if (staged) {
-        if (fast) walk_fast_staged<RD, WR, false>(smem_addr(sprog), nb, lane);
-        else walk<false, RD, WR, false>(sprog, nb, V, lane);
+        if (fast) walk_fast_staged<RD, WR, false, W>(smem_addr(sprog), nb, lane, warp);
+        else walk<false, RD, WR, false, W>(sprog, nb, V, lane, warp);
     } else {
-        if (fast) walk<true, RD, WR, false>(gw, nb, V, lane);
-        else walk<false, RD, WR, false>(gw, nb, V, lane);
+        if (fast) walk<true, RD, WR, false, W>(gw, nb, V, lane, warp);
+        else walk<false, RD, WR, false, W>(gw, nb, V, lane, warp);
     }
-    __syncwarp();      // the iteration's writes before the next one reads them
+    // the iteration's writes before the next one reads them
+    if (W == 1) __syncwarp();
+    else __syncthreads();
 }
 
 // K synchronous iterations of recurrent lane programs (records of
@@ -1075,20 +1082,20 @@ __device__ __forceinline__ void rnn_iteration(const unsigned char *sprog, const 
 // non-input node from iteration k-1's values (tile k mod 2 -> tile (k+1)
 // mod 2); the outputs are read from tile K mod 2.  Staging, inputs and
 // error handling as in lanes_kernel.
-template <bool PDL>
-__global__ void __launch_bounds__(32) lanes_rnn_kernel(const LanesArgs a, int K)
+template <bool PDL, int W>
+__global__ void __launch_bounds__(32 * W) lanes_rnn_kernel(const LanesArgs a, int K)
 {
     unsigned char *sm = lane_sm;
     float *V = reinterpret_cast<float *>(sm + kLaneBar);
     unsigned char *sprog = sm + kLaneBar + lanes_rnn_tile_bytes(a.N);
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned char *gw = a.lanes + a.warp_base + (size_t)blockIdx.x * a.warp_stride;
     const uint4 wh = __ldg(reinterpret_cast<const uint4 *>(gw));
     const int2 li = __ldg(reinterpret_cast<const int2 *>(gw + 16) + lane);
     const uint32_t bytes = wh.y;
     const bool staged = bytes <= a.cap;
     const uint32_t bar = smem_addr(sm);
-    if (staged && lane == 0) {
+    if (staged && threadIdx.x == 0) {
         mbar_init(bar, 1);
         mbar_arrive_expect_tx(bar, bytes);
         bulk_g2s(smem_addr(sprog), gw, bytes, bar);
@@ -1096,11 +1103,10 @@ __global__ void __launch_bounds__(32) lanes_rnn_kernel(const LanesArgs a, int K)
     const int g = li.x;
     // both tiles zero (non-input nodes start at 0; the zero slots), the one
     // slots 1; tiles are block-private, so this overlaps the previous kernel
-    for (int i = lane; i < (a.N + 3) * 64; i += 32) V[i] = 0.0f;
-    V[(a.N + 1) * 64 + lane] = 1.0f;
-    V[(a.N + 1) * 64 + 32 + lane] = 1.0f;
+    for (int i = threadIdx.x; i < (a.N + 3) * 64; i += 32 * W)
+        V[i] = i / 64 == a.N + 1 ? 1.0f : 0.0f;
     if constexpr (PDL) {
-        if (g >= 0 && a.I > 0 && lane < kLaneJ) {
+        if (warp == 0 && g >= 0 && a.I > 0 && lane < kLaneJ) {
             const char *p0 = reinterpret_cast<const char *>(a.x + (size_t)g * a.I);
             const char *p1 = p0 + 4u * (uint32_t)a.I - 1;
             for (const char *p = p0; p <= p1; p += 128) prefetch_l2(p);
@@ -1109,34 +1115,31 @@ __global__ void __launch_bounds__(32) lanes_rnn_kernel(const LanesArgs a, int K)
         pdl_wait();
         pdl_trigger();
     }
-    __syncwarp();
-    load_inputs<64, true>(a.x, a.x + (size_t)a.pop * a.I, g, a.I, lane, V);
-    bool ok = true;
-    if (staged) {
-        __syncwarp();
-        ok = __all_sync(0xffffffffu, mbar_wait(bar, 0));
-        if (!ok) {
-            if (lane == 0) atomicOr(&g_lanes_error, kErrWaitExpired);
-            mbar_wait(bar, 0);
-        }
+    __syncthreads();                     // the tiles are cleared, the barrier is initialised
+    if (warp == 0) load_inputs<64, true>(a.x, a.x + (size_t)a.pop * a.I, g, a.I, lane, V);
+    bool ok = !staged || mbar_wait(bar, 0);
+    ok = __syncthreads_and(ok) != 0;     // one verdict for the block: its warps meet at every iteration
+    if (!ok) {
+        if (threadIdx.x == 0) atomicOr(&g_lanes_error, kErrWaitExpired);
+        mbar_wait(bar, 0);
     }
-    __syncwarp();
     const int nb = (int)(wh.x & 0xffffu);
     if (!(wh.z & kWarpRecurrent)) ok = false;   // a feedforward program: its offsets index one tile
     if (ok) {
         const bool fast = (wh.z & kWarpFast) != 0;
         for (int k = 0; k + 1 < K; k += 2) {
-            rnn_iteration<0u, 128u>(sprog, gw, staged, fast, nb, V, lane);
-            rnn_iteration<128u, 0u>(sprog, gw, staged, fast, nb, V, lane);
+            rnn_iteration<0u, 128u, W>(sprog, gw, staged, fast, nb, V, lane, warp);
+            rnn_iteration<128u, 0u, W>(sprog, gw, staged, fast, nb, V, lane, warp);
         }
-        if (K & 1) rnn_iteration<0u, 128u>(sprog, gw, staged, fast, nb, V, lane);
+        if (K & 1) rnn_iteration<0u, 128u, W>(sprog, gw, staged, fast, nb, V, lane, warp);
     }
     if (g >= 0) {
         float *yg = a.y + (size_t)g * a.O;
         const bool nan_out = !ok || (li.y & (int)(kLaneError | kLaneUnordered));
         const float qnan = __int_as_float(0x7fc00000);
         const int fin = (K & 1) ? 32 : 0;
-        for (int j = lane / kLaneJ; j < a.O; j += kLaneG) yg[j] = nan_out ? qnan : V[(a.I + j) * 64 + fin + lane];
+        for (int j = warp * kLaneG + lane / kLaneJ; j < a.O; j += kLaneG * W)
+            yg[j] = nan_out ? qnan : V[(a.I + j) * 64 + fin + lane];
     }
 }
 
@@ -1196,17 +1199,46 @@ int make_lanes_args(const void *lanes, int32_t pop, const neat_dims &d, const fl
     return NEAT_OK;
 }
 
+// Warps that share a recurrent warp program's beats (any number gives the
+// same bits), for a launch of `programs` blocks of `smem` bytes.  One warp
+// leaves the schedulers idle: 8 iterations, 50 nodes and 200 connections,
+// 1 000 genomes 12.9 us, with two warps 9.7, with four 8.3; 128 nodes and 512
+// connections 33.7, 22.0, 14.8; 10 000 genomes of 100 nodes 44.6, 34.3, 28.7.
+// Four: up to 2.5 blocks per SM, and where no more than four fit on one.  With
+// more blocks a full SM is busy with fewer warps each, and two are as good or
+// better: 9 500 genomes of 40 nodes 13.3, 12.8, 14.2; 10 000 of 24 nodes 9.4,
+// 8.7, 9.1; of 48 nodes 15.8, 14.4, 14.8.  One, where more than four blocks per
+// SM are launched and an SM has room for a part of the next launch's share:
+// overlapping launches then spread over the SMs unevenly, which costs most
+// when a block keeps its SM busy (10 000 of 32 nodes 12.0, 12.8, 15.0).
+int rnn_warps(int programs, size_t smem)
+{
+    int dev = 0, sms = 152, smem_sm = 228 * 1024;
+    if (cudaGetDevice(&dev) == cudaSuccess) {
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    }
+    const long fit = smem_sm / (long)(smem + 1024u);   // 1 KB reserved per block
+    if (2L * programs <= 5L * sms || fit <= 4) return 4;
+    const long need = (programs + sms - 1L) / sms;
+    return need > 4 && fit > need + 1 && fit < 2 * need - 1 ? 1 : 2;
+}
+
 int launch_lanes_rnn(const LanesArgs &a, int warps, int K, bool pdl, cudaStream_t s)
 {
     if (warps == 0) return NEAT_OK;
     const size_t smem = kLaneBar + lanes_rnn_tile_bytes(a.N) + a.cap;
-    auto f = pdl ? lanes_rnn_kernel<true> : lanes_rnn_kernel<false>;
+    const int share = rnn_warps(warps, smem);
+    using Kern = void (*)(const LanesArgs, int);
+    const Kern f = share == 4   ? (pdl ? lanes_rnn_kernel<true, 4> : lanes_rnn_kernel<false, 4>)
+                   : share == 2 ? (pdl ? lanes_rnn_kernel<true, 2> : lanes_rnn_kernel<false, 2>)
+                                : (pdl ? lanes_rnn_kernel<true, 1> : lanes_rnn_kernel<false, 1>);
     int rc = allow_dynamic_smem(reinterpret_cast<const void *>(f), smem,
                                 "neat_forward_lanes_recurrent: shared memory per block");
     if (rc) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)warps);
-    cfg.blockDim = dim3(32);
+    cfg.blockDim = dim3((unsigned)(32 * share));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
