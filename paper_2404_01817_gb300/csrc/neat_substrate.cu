@@ -144,11 +144,17 @@ __global__ void __launch_bounds__(kSubThreads) substrate_kernel(const SubArgs a)
             const int c = c0 + col_in_pass;
             if (grp < a.groups && c < ncols) {
                 // accumulators in pairs: of columns, or of vectors where a thread
-                // has one column; a lone vector's single column stays scalar
-                constexpr bool kPairs = NB * VEC > 1;
+                // has one column and sixteen.  With one column and fewer vectors
+                // the pairs of vectors cost registers (125 instead of 48 at
+                // eight) and what they save is not what bounds it: scalar sums
+                // (427 substrates of 15 x 15, 8 vectors: 102 us, 151 in pairs)
+                constexpr bool kPairs = VEC > 1 || NB > 8;
                 constexpr int kAcc = kPairs ? NB * VEC / 2 : 1;
                 f2 as[kAcc], ac[kAcc];
-                float s1f = 0.0f, c1f = 0.0f;
+                constexpr int kOne = kPairs ? 1 : NB;
+                float s1f[kOne], c1f[kOne];
+#pragma unroll
+                for (int b = 0; b < kOne; ++b) s1f[b] = c1f[b] = 0.0f;
 #pragma unroll
                 for (int k = 0; k < kAcc; ++k) as[k] = ac[k] = 0ull;
                 const int s0 = grp * slice, s1 = min(R, s0 + slice);
@@ -157,7 +163,8 @@ __global__ void __launch_bounds__(kSubThreads) substrate_kernel(const SubArgs a)
                 for (int s = s0; s < s1; ++s) {
                     const V wv = __ldg(col + (size_t)s * ncols);
                     if constexpr (!kPairs) {
-                        dot2_step(s1f, c1f, cur[s], VecT<VEC>::get(wv, 0));
+#pragma unroll
+                        for (int b = 0; b < NB; ++b) dot2_step(s1f[b], c1f[b], cur[b * R + s], VecT<VEC>::get(wv, 0));
                     } else if constexpr (VEC == 1) {
                         const f2 w2 = pack2(VecT<VEC>::get(wv, 0), VecT<VEC>::get(wv, 0)), nw2 = neg2(w2);
 #pragma unroll
@@ -184,7 +191,8 @@ __global__ void __launch_bounds__(kSubThreads) substrate_kernel(const SubArgs a)
                     pc[((size_t)grp * NB + b) * R + c * VEC + v] = err;
                 };
                 if constexpr (!kPairs) {
-                    put(0, 0, s1f, c1f);
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) put(b, 0, s1f[b], c1f[b]);
                 } else {
 #pragma unroll
                     for (int k = 0; k < kAcc; ++k) {
