@@ -474,9 +474,10 @@ constexpr uint32_t kNoBar = 0xffffffffu;
 //   the value tile, at least one column of the genome's nodes (a genome with
 //   more nodes than the tile has rows takes fewer columns at a time).
 // False, with nothing evaluated, when the record is longer than rec_limit
-// bytes (the part that was copied).  PAIRS: two columns per thread (tile at
+// bytes (the part that was copied), or (WHOLE: all columns at once) has more
+// nodes than the tile has rows.  PAIRS: two columns per thread (tile at
 // least 2, at most 2 G; vcap at least two columns).
-template <bool T1, bool PAIRS = false>
+template <bool T1, bool PAIRS = false, bool WHOLE = false>
 __device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t bar, volatile int *flag, int G,
                                          int gi, int lane, const float *__restrict__ xb, float *__restrict__ yb,
                                          int I, int O, int bt, int tile, int lg_split, int vcap, uint32_t rec_limit,
@@ -506,11 +507,14 @@ __device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t b
     }
     if (h1.x > rec_limit) return false;
     const uint16_t *io = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.w);
-    if constexpr (!T1)
+    if constexpr (!T1 && WHOLE) {
+        if (((int)(h0.x & 0xffffu) << lgT) > vcap) return false;
+    } else if constexpr (!T1)
         while (lgT > (PAIRS ? 1 : 0) && ((int)(h0.x & 0xffffu) << lgT) > vcap) --lgT;
     const int step = T1 ? 1 : 1 << lgT;
-    for (int c0 = 0; c0 < bt; c0 += step) {                 // once, unless the nodes outgrow the tile's rows
-        const int cols = T1 ? 1 : min(bt - c0, step);
+    constexpr bool kOnce = T1 || WHOLE;
+    for (int c0 = 0; c0 < (kOnce ? 1 : bt); c0 += step) {   // once, unless the nodes outgrow the tile's rows
+        const int cols = T1 ? 1 : WHOLE ? bt : min(bt - c0, step);
         const int ni = cols * I;
         if (c0 > 0) {
             group_sync(G, gi);                              // the last columns' outputs were read

@@ -19,7 +19,7 @@
 // kernel (run_item), so results match neat_forward bit for bit.
 //
 // Four populations of 2048 genomes (up to 16, 64, 256 and 1024 nodes), 64
-// inputs each: 189 us a step with compact records (509 us without), the 49 us
+// inputs each: 182 us a step with compact records (509 us without), the 49 us
 // copy included.
 #include <algorithm>
 #include <climits>
@@ -296,9 +296,9 @@ plan_kernel(const BucketDev *__restrict__ buckets, int nb, int item_lo, int item
             const bool t1 = d.tile == 1;
             bool done = false;
             if (staged)
-                done = t1 ? run_item<true>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split,
+                done = t1 ? run_item<true, false, true>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split,
                                            vcap, limit, &g_plan_error)
-                          : run_item<false>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, vcap,
+                          : run_item<false, false, true>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, vcap,
                                             limit, &g_plan_error);
             if (!done) {
                 const uint4 *grec = reinterpret_cast<const uint4 *>(d.rec + (size_t)g * d.stride);
@@ -828,20 +828,25 @@ int read_headers(neat_plan *P, bool compact, cudaStream_t s, std::vector<std::ve
     return NEAT_OK;
 }
 
-// Whether the nodes saved are worth the copy that every call makes: a warp's
-// work on one node for 32 columns is about 130 instructions, so the 8 us or
-// so that the copy takes are 50 000 of them at the rate the steps run at.
+// Whether the nodes saved are worth the copy that every call makes.  A warp
+// takes a node for 32 columns, or several nodes for fewer, in about 130
+// instructions; 100 000 of those are what the copy and its wait cost.  Small
+// batches save little per node: 248 genomes each of 56 to 441 rows and 8
+// vectors, 32 us a step as they are and 49 with copies; 425 of 26 to 284 rows
+// and 3 vectors 32 and 47; 1 669 of 20 to 509 rows and 3 vectors 59 and 62.
+// (Some small batches of large genomes would gain and stay as they are: 1 723
+// of 216 and 700 rows and 2 vectors, 94 and 69.)
 bool compact_pays(const neat_plan *P, const std::vector<std::vector<uint32_t>> &full,
                   const std::vector<std::vector<uint32_t>> &compact)
 {
     double saved = 0.0;
     for (size_t p = 0; p < full.size(); ++p) {
         const int batch = P->pops[p].batch;
-        const double per_node = batch <= 1 ? 0.25 : (double)((batch + 31) / 32);
+        const double per_node = batch > 16 ? (double)((batch + 31) / 32) : std::max(4, 1 << lg(batch)) / 32.0;
         for (size_t g = 0; g * 8 < full[p].size(); ++g)
             saved += per_node * ((double)(full[p][g * 8] & 0xffffu) - (double)(compact[p][g * 8] & 0xffffu));
     }
-    return saved > 50000.0;
+    return saved > 100000.0;
 }
 
 }  // namespace
