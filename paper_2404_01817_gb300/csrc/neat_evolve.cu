@@ -8,8 +8,9 @@
 // float normals give the perturbations.
 //
 // GB300 mapping: one warp per genome up to 128 node rows and 512 connection
-// rows (mutate_warp_kernel, crossover_warp_kernel), one block per genome
-// beyond.  The block forms work in place on the population tensors: the node
+// rows (mutate_warp_kernel, crossover_warp_kernel; above 288 and 208
+// connection rows for large populations only), else one block per genome.
+// The block forms work in place on the population tensors: the node
 // keys and the connections' (in, out, enabled) columns are kept in shared
 // memory while the four structural steps run one after another (block-wide
 // counts, rank selection by a block scan, first-free-row searches, and for
@@ -964,7 +965,10 @@ extern "C" int neat_mutate(float *nodes_dev, float *conns_dev, int32_t pop, neat
     for (int i = 0; i < 8; ++i) a.act_opt[i] = m->activation_options[i];
     for (int i = 0; i < 4; ++i) a.agg_opt[i] = m->aggregation_options[i];
     a.feedforward = m->feedforward != 0;
-    if (a.N <= kWarpNodes && a.C <= kWarpConns) {
+    // above 288 rows a lone warp's chain is the longer one until there are
+    // genomes enough to hide it (97 / 388 rows: 500 genomes 17.5 us, 14.7 by
+    // blocks; 2000: 17.3 and 24.0)
+    if (a.N <= kWarpNodes && a.C <= kWarpConns && (a.C <= 288 || pop >= 1500)) {
         const int warps = pop > 4 * 152 ? 4 : 1;
         const size_t bytes = (size_t)warps * mut_warp_layout(a.N, a.C, a.Np2).total;
         const int rw = allow_dynamic_smem(reinterpret_cast<const void *>(mutate_warp_kernel), bytes,
@@ -1012,7 +1016,10 @@ extern "C" int neat_crossover(const float *nodes_dev, const float *conns_dev, in
     a.C = d.max_conns;
     a.Np2 = pow2_at_least(a.N);
     a.Cp2 = pow2_at_least(a.C > 0 ? a.C : 1);
-    if (a.N <= kWarpNodes && a.C <= kWarpConns) {
+    // the same from 208 rows on, with the longer chain of lookups (72 / 289
+    // rows: 1000 children 20.7 us, 12.7 by blocks; 4000: 24.8 and 30.6; 128 /
+    // 512: 4000 51.7 and 50.8)
+    if (a.N <= kWarpNodes && a.C <= kWarpConns && (a.C <= 208 || n_children >= 12 * a.C)) {
         const int warps = n_children > 4 * 152 ? 4 : 1;
         const size_t bytes = (size_t)warps * cross_warp_layout(a.N, a.Np2, a.Cp2).total;
         const int rw = allow_dynamic_smem(reinterpret_cast<const void *>(crossover_warp_kernel), bytes,
