@@ -196,8 +196,8 @@ NEAT_API int neat_transform(const float *nodes_dev, const float *conns_dev, int3
  *   inputs_dev       f32 [pop][batch][I]
  *   outputs_dev      f32 [pop][batch][O] (written; NaN for genomes with an error bit)
  * The launch shape is chosen from (pop, dims, batch), as neat_default_launch
- * says; batches above 32 are evaluated two input vectors per thread where the
- * genomes' values are small enough, and one vector for many large genomes reads
+ * says; 33 to 64 vectors for many large genomes are evaluated two per thread
+ * where the genomes' values are small enough, and one vector for many large genomes reads
  * the records where they lie.  The results do not depend on it.
  * Errors: NEAT_EINVAL, NEAT_ECUDA.
  */

@@ -452,10 +452,15 @@ extern "C" int neat_forward_ex(const void *transformed_dev, int32_t pop, neat_di
         const cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "forward: launch");
     }
-    if (!launch_host && batch > 32) {
+    if (!launch_host && batch > 32 && batch <= 64 && d.max_nodes >= kMinPairNodes && pop >= kMinPairPop) {
         // two columns per thread in tiles of 64, where four such groups fit an
-        // SM.  1001 genomes of 101 / 403 rows and 37 vectors: 51 -> 46 us with
-        // the transform (one tile of 37 instead of tiles of 32 and 5).  (In the
+        // SM, there are genomes enough to fill it and a level has nodes enough
+        // for the fewer threads (a launch, 40 vectors, sum and tanh: 1200
+        // genomes of 50 rows 17 us in tiles of 32 and 19 in pairs, 300 of 101
+        // rows 18 and 19, 2400 of 101 rows 51 and 45; 67 vectors, whose second
+        // tile is nearly empty: 73 and 95).  1001 genomes of 101 / 403 rows and
+        // 37 vectors, mixed activations and aggregations: 51 -> 46 us with the
+        // transform (one tile of 37 instead of tiles of 32 and 5).  (In the
         // plan's kernel, whose registers it overran, the same shapes took 195
         // instead of 189 us a step)
         neat_launch W = L;

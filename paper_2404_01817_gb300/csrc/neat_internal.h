@@ -60,6 +60,7 @@ constexpr size_t kMaxGroupSmem = 200u * 1024u;
 // The same for a tile of 64 columns, two per thread: beyond, fewer than four
 // groups share an SM and the tile of 32 is the better one.
 constexpr size_t kMaxPairGroupSmem = 48u * 1024u;
+constexpr int kMinPairNodes = 96, kMinPairPop = 1000;
 
 // Threads per tile row for a genome of up to n nodes and a batch of several
 // input vectors: about one per 32 nodes (a level of a large genome holds
