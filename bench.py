@@ -371,11 +371,10 @@ def measure_batched(args):
     plain()
     ms_p = timed_events(plain, max(1, min(args.steps, 5)), stream)
     gf = sum(p.pop for p in pops) * B * S
-    # algorithmic bytes of one step: every record once, the step's inputs and outputs
-    alg = 0
-    for p, dd in zip(pops, descs):
-        hdr = dd["transformed"][:p.pop * neat.neat_record_stride(dd["dims"])].view(p.pop, -1)[:, :32].cpu().numpy()
-        alg += int(hdr.view(np.uint32)[:, 4].astype(np.int64).sum()) + 4 * p.pop * B * (p.num_inputs + p.num_outputs)
+    # algorithmic bytes of one step: the nodes and connections the outputs
+    # depend on, the step's inputs and outputs
+    alg = sum(genome_forward_bytes(needed_population(p))[0] + 4 * p.pop * (B - 1) * (p.num_inputs + p.num_outputs)
+              for p in pops)
     t_step = statistics.median(ms_b) / 1e3 / S
     peak, src = measured_peaks()
     line = {"metric": "genome-forwards/s (batched uneven: 4 pops x 2048, Nmax 16/64/256/1024, B=64)",
@@ -387,14 +386,42 @@ def measure_batched(args):
             "plan": plan.describe(), "clocks": clocks.summary(),
             "roofline": {"bound": "hbm", "achieved": alg / t_step / 1e9, "peak": peak, "unit": "GB/s",
                          "frac": alg / t_step / 1e9 / peak, "traffic": None, "peak_source": src,
-                         "note": "plan kernel per step; algorithmic bytes = every record once + inputs + outputs. "
-                                 "The large buckets are bound by shared-memory gathers (4 B per edge per input "
+                         "note": "plan kernel per step (the compact copy of the records once per graph); "
+                                 "algorithmic bytes = 16 B per node and 6 B per connection that the outputs "
+                                 "depend on, + inputs + outputs. The large buckets are bound by shared-memory gathers (4 B per edge per input "
                                  "vector) and FP32/SFU issue, not HBM"},
             "gpu_launches": args.steps * S,
             "parity": {"max_scaled_error": max(errs), "per_population": errs,
                        "compared": "step 0, 16 genomes x 64 inputs per population vs the FP64 oracle"}}
     plan.close()
     return line
+
+
+def needed_population(pop):
+    """The population without what no output depends on (node rows and their
+    incoming connections as NaN): what a forward has to read and compute, for
+    the rooflines.  For genomes whose node keys are their rows."""
+    from paper_2404_01817_gb300 import workloads as W
+    c = pop.conns
+    on = ~np.isnan(c[:, :, :3]).any(2) & (np.nan_to_num(c[:, :, 2]) != 0)
+    g, k = np.nonzero(on)
+    src, dst = c[g, k, 0].astype(np.int64), c[g, k, 1].astype(np.int64)
+    need = np.zeros(pop.nodes.shape[:2], dtype=bool)
+    need[:, pop.num_inputs:pop.num_inputs + pop.num_outputs] = True
+    while True:
+        before = int(need.sum())
+        m = need[g, dst]
+        need[g[m], src[m]] = True
+        if int(need.sum()) == before:
+            break
+    need[:, :pop.num_inputs] = True
+    nodes, conns = pop.nodes.copy(), pop.conns.copy()
+    nodes[~need] = np.nan
+    gone = np.ones(on.shape, dtype=bool)
+    keep = need[g, dst]
+    gone[g[keep], k[keep]] = False
+    conns[gone] = np.nan
+    return W.Population(nodes, conns, pop.num_inputs, pop.num_outputs)
 
 
 def run_cppn(args):
@@ -436,13 +463,16 @@ def measure_cppn(args):
     flip = (got == 0) != (ref == 0)
     flips_ok = bool(np.all(np.abs(np.abs(raw[flip]) - 0.2) <= 1e-5 * np.maximum(1, np.abs(raw[flip]))))
     _, _, err = oracle_error(got[~flip], ref[~flip])
-    hdr = rec.view(1000, -1)[:, :32].cpu().numpy().view(np.uint32)
-    edges = hdr[:, 1].astype(np.int64)
-    nonin = (hdr[:, 0] & 0xFFFF).astype(np.int64) - 5
+    # what a query needs: the nodes and connections that its output depends on
+    sub = needed_population(pop)
+    edges = (~np.isnan(sub.conns[:, :, 0])).sum(1).astype(np.int64)
+    nonin = (~np.isnan(sub.nodes[:, :, 0])).sum(1).astype(np.int64) - 5
     q = 1000 * 131072
     t = statistics.median(ms) / 1e3
     tq = statistics.median(ms_q) / 1e3
-    flops = 131072 * int((2 * edges + 2 * nonin).sum())       # one FMA per edge, bias/response FMA per node
+    # one FMA per edge, bias/response FMA per node; the two blocks of a genome
+    # have the same queries (no layer coordinate), evaluated once
+    flops = 65536 * int((2 * edges + 2 * nonin).sum())
     cs = clocks.summary()
     sm_mhz = cs["sm_mhz"] or cs["sm_max_mhz"] or 2070.0
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
@@ -451,11 +481,12 @@ def measure_cppn(args):
             "value": q / t, "unit": "queries/s", "n_gpus": 1, "steps": max(args.steps, 50), "warmup": args.warmup,
             "ms_per_step": statistics.median(ms), "higher_is_better": True, "dtype": "f32", "data": "synthetic",
             "config": {"workload": "CPPN", "genomes": 1000, "queries_per_genome": 131072,
+                       "distinct_queries_per_genome": 65536,
                        "l2": "no flush: 524 MB of weights written per step, larger than L2"},
             "query_kernel_ms": tq * 1e3,
             "roofline": {"bound": "alu", "achieved": flops / tq / 1e12, "peak": fp32_peak, "unit": "TFLOP/s",
                          "frac": flops / tq / 1e12 / fp32_peak,
-                         "note": f"FMA flops of the edges and node rule against {sms} SMs x 128 FP32 lanes x 2 at "
+                         "note": f"FMA flops of the distinct queries' needed edges and nodes against {sms} SMs x 128 FP32 lanes x 2 at "
                                  "the sampled clock; the transcendental activations (sin, exp) are not counted"},
             "parity": {"max_scaled_error": err, "threshold_flips_at_boundary_only": flips_ok,
                        "threshold_flips": int(flip.sum()), "compared": "2000 random queries vs the FP64 oracle"},
@@ -814,7 +845,7 @@ def run_evolve(args):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": None, "peak_source": src,
                          "note": "mutation kernel: child tensors read + written and its random inputs read; "
-                                 "one block per genome runs the structural steps with block barriers, so it is "
+                                 "one warp per genome runs the structural steps one after another, so it is "
                                  "latency-bound"},
             "cpu_baseline": {"value": idx.size / dt_all, "unit": "genomes/s", "cores": cores, "kind": "oracle",
                              "sample": f"{idx.size} children: crossover + mutation, FP64 C oracle, {cores} threads "
@@ -1356,7 +1387,8 @@ def main():
     link_floor = world * POP * S / max(t_up, t_dn)
 
     # ---- roofline of the forward kernel: algorithmic bytes per launch
-    alg_bytes, n_nodes, n_edges = genome_forward_bytes(pop)
+    alg_bytes, n_nodes, n_edges = genome_forward_bytes(needed_population(pop))
+    all_bytes, all_nodes, all_edges = genome_forward_bytes(pop)
     hdr = rec.view(POP, -1)[:, :32].cpu().numpy().view(np.uint32)
     record_bytes = int(hdr[:, 4].astype(np.int64).sum())                  # used bytes of every record
     program_bytes = lane_program_bytes(lanes, info)
@@ -1439,9 +1471,10 @@ def main():
                      "peak_kind": f"{peak_kind} hbm_gbs",
                      "kernel": "lanes_kernel (batched form, per launch, graph-amortised)",
                      "alg_bytes_per_launch": alg_bytes,
-                     "alg_bytes_rule": "per genome 16 B x present nodes + 6 B x enabled connections, + 4 B x "
-                                       "(inputs + outputs); counted from the generated tensors",
-                     "present_nodes": n_nodes, "enabled_connections": n_edges,
+                     "alg_bytes_rule": "per genome 16 B x nodes + 6 B x enabled connections that the outputs "
+                                       "depend on, + 4 B x (inputs + outputs); counted from the generated tensors",
+                     "needed_nodes": n_nodes, "needed_connections": n_edges,
+                     "present_nodes": all_nodes, "enabled_connections": all_edges, "bytes_of_all_present": all_bytes,
                      "program_bytes_per_launch": program_bytes,
                      "record_bytes": record_bytes,
                      "l2_traffic_over_alg": (l2_traffic / alg_bytes) if l2_traffic else None},
