@@ -814,7 +814,22 @@ __device__ __forceinline__ void load_beat_head(BeatState &st, uint4 ne, uint32_t
     for (int t = 0; t < kHeadRows; ++t) st.q[t] = lds_quad((uint32_t)t < st.mt ? st.base + (uint32_t)t * kRowBytes : ra);
 }
 
-// The warp's beats from b up to `end`, every one with T trips (T even, known at
+// A lone warp counts a run's beats; warps that share it step to its end (the
+// counted form for both: 10 000 recurrent genomes of 20 nodes 8.5 -> 9.6 us a
+// step; the stepped form for both: the Ant step 3.67 -> 3.72 us).
+template <int W, typename F>
+__device__ __forceinline__ void each_beat(const F &beat, int &b, int len, int end)
+{
+    if constexpr (W == 1) {
+        int c = b;
+        for (int i = 0; i < len; ++i, ++c) beat(c);
+    } else {
+        for (; b < end; b += W) beat(b);
+    }
+}
+
+// A run's beats from b on (`len` of them; where warps share it, this one's
+// before `end`), every one with T trips (T even, known at
 // compile time; T = 0: nodes without edges).  Per beat: rows kHeadRows..T-1
 // loaded (the first rows are in the state), then the values and the fused
 // multiply-adds in trip order per partial; the next beat's head (entry and
@@ -822,9 +837,10 @@ __device__ __forceinline__ void load_beat_head(BeatState &st, uint4 ne, uint32_t
 // every column of the genome and the warp barrier.  A lane past its own
 // quads reads the padding quad at `ra`.
 template <int T, uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true, int W = 1>
-__device__ __forceinline__ void run_beats(BeatState &st, int &b, int end, int nb, uint32_t na, uint32_t ra, int lane)
+__device__ __forceinline__ void run_beats(BeatState &st, int &b, int len, int end, int nb, uint32_t na, uint32_t ra,
+                                          int lane)
 {
-    for (; b < end; b += W) {
+    auto beat = [&](int b) {
         const uint4 nn = b + W < nb ? lds_u4(na + 512u * (uint32_t)(b + W)) : st.ne;
         float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;
         if (T > 0) {
@@ -844,15 +860,16 @@ __device__ __forceinline__ void run_beats(BeatState &st, int &b, int end, int nb
         for (int m = 0; m < kLaneG; ++m)
             tile_st(((dst & ~127u) + WR) | ((uint32_t)((lane + m * kLaneJ) & 31) << 2), v);
         if (SYNC) __syncwarp();
-    }
+    };
+    each_beat<W>(beat, b, len, end);
 }
 
 // The same for any even T above 8 (trip pairs in a loop after the head rows).
 template <uint32_t RD = 0, uint32_t WR = 0, bool SYNC = true, int W = 1>
-__device__ __forceinline__ void run_beats_any(BeatState &st, int T, int &b, int end, int nb, uint32_t na, uint32_t ra,
-                                              int lane)
+__device__ __forceinline__ void run_beats_any(BeatState &st, int T, int &b, int len, int end, int nb, uint32_t na,
+                                              uint32_t ra, int lane)
 {
-    for (; b < end; b += W) {
+    auto beat = [&](int b) {
         const uint4 nn = b + W < nb ? lds_u4(na + 512u * (uint32_t)(b + W)) : st.ne;
         float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;
 #pragma unroll
@@ -872,7 +889,8 @@ __device__ __forceinline__ void run_beats_any(BeatState &st, int T, int &b, int 
         for (int m = 0; m < kLaneG; ++m)
             tile_st(((dst & ~127u) + WR) | ((uint32_t)((lane + m * kLaneJ) & 31) << 2), v);
         if (SYNC) __syncwarp();
-    }
+    };
+    each_beat<W>(beat, b, len, end);
 }
 
 // The fast form (every node sums and applies tanh) of a warp program staged
@@ -892,19 +910,29 @@ __device__ __forceinline__ void walk_fast_staged(uint32_t P, int nb, int lane, i
     if (warp >= nb) return;
     BeatState st;
     load_beat_head(st, lds_u4(na + 512u * (uint32_t)warp), ra);
-    int b = warp;                                     // the warp's next beat
-    for (int run = 0; run < nb;) {
-        const uint32_t e = lds_u32(sa + 4u * (uint32_t)run);
-        const int T = (int)(e & 0xffffu);
-        run += max(1, (int)(e >> 16));
-        const int end = min(run, nb);
+    auto beats = [&](int T, int &b, int len, int end) {
         switch (T) {
-        case 0: run_beats<0, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
-        case 2: run_beats<2, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
-        case 4: run_beats<4, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
-        case 6: run_beats<6, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
-        case 8: run_beats<8, RD, WR, SYNC, W>(st, b, end, nb, na, ra, lane); break;
-        default: run_beats_any<RD, WR, SYNC, W>(st, T, b, end, nb, na, ra, lane);
+        case 0: run_beats<0, RD, WR, SYNC, W>(st, b, len, end, nb, na, ra, lane); break;
+        case 2: run_beats<2, RD, WR, SYNC, W>(st, b, len, end, nb, na, ra, lane); break;
+        case 4: run_beats<4, RD, WR, SYNC, W>(st, b, len, end, nb, na, ra, lane); break;
+        case 6: run_beats<6, RD, WR, SYNC, W>(st, b, len, end, nb, na, ra, lane); break;
+        case 8: run_beats<8, RD, WR, SYNC, W>(st, b, len, end, nb, na, ra, lane); break;
+        default: run_beats_any<RD, WR, SYNC, W>(st, T, b, len, end, nb, na, ra, lane);
+        }
+    };
+    if constexpr (W == 1) {
+        for (int b = 0; b < nb;) {
+            const uint32_t e = lds_u32(sa + 4u * (uint32_t)b);
+            const int T = (int)(e & 0xffffu), len = max(1, (int)(e >> 16));
+            beats(T, b, len, nb);
+            b += len;
+        }
+    } else {
+        int b = warp;                                 // the warp's next beat
+        for (int run = 0; run < nb;) {
+            const uint32_t e = lds_u32(sa + 4u * (uint32_t)run);
+            run += max(1, (int)(e >> 16));
+            beats((int)(e & 0xffffu), b, 0, min(run, nb));
         }
     }
 }
