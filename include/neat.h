@@ -612,7 +612,10 @@ typedef struct neat_substrate {
 
 /* weights_dev: f32 [pop][layers-1][res*res][res*res] (written; NaN for
  * genomes with an error bit).  d must have num_inputs = 5, num_outputs = 1
- * and max_nodes <= 160.  Errors: NEAT_EINVAL, NEAT_ECUDA. */
+ * and max_nodes <= 160.  Records of neat_transform_recurrent, which hold no
+ * order, are evaluated once in node row order: the same weights where every
+ * node that the output depends on has a later row than the non-input nodes it
+ * reads, else NaN.  Errors: NEAT_EINVAL, NEAT_ECUDA. */
 NEAT_API int neat_cppn_query(const void *transformed_dev, int32_t pop, neat_dims d, neat_substrate sub,
                              float threshold, float *weights_dev, void *stream);
 

@@ -179,6 +179,14 @@ __device__ __forceinline__ void fold_edges(const typename Edge<WIDE>::T *__restr
         out[j] = agg_combine(AGG, agg_combine(AGG, q[0][j], q[1][j]), agg_combine(AGG, q[2][j], q[3][j]));
 }
 
+// NaN for the pairs [q0, qend) of every weight block of a genome.
+__device__ __forceinline__ void write_nan(float *out, const CppnArgs &a, int q0, int qend)
+{
+    for (int l = 0; l < a.blocks; ++l)
+        for (int q = q0 + (int)threadIdx.x; q < qend; q += blockDim.x)
+            out[(size_t)l * a.pairs + q] = __int_as_float(0x7fc00000);
+}
+
 template <bool WIDE>
 __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
 {
@@ -186,7 +194,7 @@ __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
     __shared__ uint64_t bar_mem;
     __shared__ float coord[256];
     __shared__ uint8_t need[kCppnMaxNodes], slot_of[kCppnMaxNodes];
-    __shared__ int failed, n_prog;
+    __shared__ int failed, n_prog, unordered;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
     const int g = (int)(blockIdx.x / a.chunks);
     const int q0 = (int)(blockIdx.x - (unsigned)g * a.chunks) * a.chunk;
@@ -200,7 +208,7 @@ __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
     if (tid == 0) {
         const uint32_t bytes = min(align16(__ldg(reinterpret_cast<const uint32_t *>(grec) + 4)),
                                    (uint32_t)a.rec_words * 16u);
-        failed = 0;
+        failed = unordered = 0;
         mbar_init(bar, 1);
         mbar_arrive_expect_tx(bar, bytes);
         bulk_g2s(smem_addr(srec), grec, bytes, bar);
@@ -219,8 +227,7 @@ __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
     if (failed || (h0.z & NEAT_G_ERROR_MASK)) {
         if (failed && tid == 0) atomicOr(&g_cppn_error, kErrWaitExpired);
         if (failed) mbar_wait(bar, 0);                     // let the copy land before the block's memory is released
-        for (int l = 0; l < a.blocks; ++l)
-            for (int q = q0 + tid; q < qend; q += nt) out[(size_t)l * a.pairs + q] = __int_as_float(0x7fc00000);
+        write_nan(out, a, q0, qend);
         return;
     }
     const int n_nodes = (int)(h0.x & 0xffffu), n_levels = (int)(h0.x >> 16), n_edges = (int)h0.y;
@@ -230,9 +237,29 @@ __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
     const uint16_t *io = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.w);
     const int p_out = io[5];
     if (tid < 32) {
-        // the nodes that the output depends on, from the last level back
+        // the nodes that the output depends on, from the last level back.  One
+        // level tells nothing of the order (neat_transform_recurrent's records:
+        // positions follow node rows): there, pass after pass over the nodes
+        // marked last (1; 2 once their sources are), until none is added, and
+        // a node must come after the nodes it reads
         if (lane == 0) need[p_out] = 1;
         __syncwarp();
+        for (bool more = n_levels == 1; more;) {
+            more = false;
+            for (int p = lane; p < n_nodes; p += 32) {
+                if (need[p] != 1) continue;
+                need[p] = 2;
+                const uint32_t z = nodes[p].z;
+                for (uint32_t i = z & 0xffffu, e = i + (z >> 16); i < e; ++i) {
+                    const uint32_t src = packed[i].y;
+                    if (need[src] == 0) need[src] = 1;
+                    if ((int)src >= p && (nodes[src].w & 0xffu) != kInputAct) unordered = 1;
+                    more = true;
+                }
+            }
+            __syncwarp();
+            more = __any_sync(0xffffffffu, more);
+        }
         for (int l = n_levels - 1; l > 0; --l) {
             for (int p = lev[l] + lane; p < lev[l + 1]; p += 32)
                 if (need[p]) {
@@ -258,6 +285,10 @@ __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
         if (lane == 0) n_prog = count;
     }
     __syncthreads();
+    if (unordered) {
+        write_nan(out, a, q0, qend);
+        return;
+    }
     // four columns per thread, as many threads as the rows leave room for
     const int np = n_prog;
     const int active = min(nt, (a.tile_bytes / (16 * (5 + np))) & ~31);
