@@ -67,6 +67,18 @@ struct CompactPop {
 
 constexpr int kCompactWarps = 4;
 
+// Whether a header describes a record of these sizes (a plan may be created
+// before its records are written; whatever lies there then is not followed).
+__device__ __forceinline__ bool header_holds(const uint4 &h0, const uint4 &h1, int I, int O, uint64_t stride)
+{
+    const uint32_t n = h0.x & 0xffffu, nl = h0.x >> 16, E = h0.y;
+    const uint32_t off_edge = kHeaderBytes + kNodeBytes * n, off_level = align16(off_edge + kEdgeBytes * E);
+    const uint32_t off_io = align16(off_level + 2u * (nl + 1u));
+    return n >= (uint32_t)(I + O) && n <= (uint32_t)NEAT_MAX_NODES && E <= (uint32_t)NEAT_MAX_CONNS && nl >= 1u &&
+           nl <= n && h1.y == off_edge && h1.z == off_level && h1.w == off_io &&
+           h1.x == align16(off_io + 2u * (uint32_t)(I + O)) && h1.x <= stride;
+}
+
 __global__ void __launch_bounds__(32 * kCompactWarps)
 compact_kernel(const CompactPop *__restrict__ pops, int np, const CompactPop one, int total, unsigned int *counters,
                int nc, unsigned int *largest)
@@ -91,10 +103,11 @@ compact_kernel(const CompactPop *__restrict__ pops, int np, const CompactPop one
     const int I = P.I, O = P.O;
     const uint4 h0 = __ldg(reinterpret_cast<const uint4 *>(src)), h1 = __ldg(reinterpret_cast<const uint4 *>(src) + 1);
     uint4 *out = reinterpret_cast<uint4 *>(dst);
-    if (h0.z & NEAT_G_ERROR_MASK) {
+    if ((h0.z & NEAT_G_ERROR_MASK) || !header_holds(h0, h1, I, O, P.stride)) {
+        // nothing to evaluate: outputs NaN
         if (lane == 0) {
-            out[0] = h0;
-            out[1] = h1;
+            out[0] = make_uint4(0u, 0u, h0.z & NEAT_G_ERROR_MASK ? h0.z : h0.z | NEAT_G_MISSING_IO, 0xffffu);
+            out[1] = make_uint4(kHeaderBytes, kHeaderBytes, kHeaderBytes, kHeaderBytes);
         }
         return;
     }
@@ -904,7 +917,7 @@ extern "C" int neat_plan_create(const neat_pop_desc *pops, int32_t npops, const 
         std::vector<int> slot_of_class(12, -1);
         for (int g = 0; g < pd.pop; ++g) {
             const uint32_t *h = &hdrs[p][(size_t)g * 8];
-            int n = (int)(h[0] & 0xffffu);
+            const int n = std::min((int)(h[0] & 0xffffu), pd.dims.max_nodes);
             int cls = o.size_buckets ? std::max(16, 1 << lg(std::max(n, 1))) : max_class;
             cls = std::min(cls, std::max(16, max_class));
             int key = lg(cls);
