@@ -187,6 +187,31 @@ __device__ __forceinline__ int mask_first(uint32_t mine)
     return owner * 32 + __shfl_sync(kAll, __ffs(mine) - 1, owner);
 }
 
+// Lowest present row holding a key, for keys of any size: a slot holds the key's
+// low 24 bits and a row, and a row is taken by its whole key, as in the block
+// form's table (a malformed genome's keys at or above 2^24 are nodes of their
+// own in both).  At most half the slots are taken.
+__device__ __forceinline__ void insert_row(uint32_t *tab, uint32_t mask, int shift, const float *ns, uint32_t row)
+{
+    const uint32_t key = (uint32_t)ns[5 * row], v = (key << 8) | row;
+    for (uint32_t s = slot32(key, shift);; s = (s + 1u) & mask) {
+        const uint32_t old = atomicCAS(tab + s, kFree32, v);
+        if (old == kFree32) return;
+        if ((old >> 8) == (v >> 8) && (uint32_t)ns[5 * (old & 0xffu)] == key) {
+            atomicMin(tab + s, v);
+            return;
+        }
+    }
+}
+__device__ __forceinline__ int find_row(const uint32_t *tab, uint32_t mask, int shift, const float *ns, uint32_t key)
+{
+    for (uint32_t s = slot32(key, shift);; s = (s + 1u) & mask) {
+        const uint32_t v = tab[s];
+        if (v == kFree32) return -1;
+        if ((v >> 8) == (key & 0xffffffu) && (uint32_t)ns[5 * (v & 0xffu)] == key) return (int)(v & 0xffu);
+    }
+}
+
 struct MutWarpLayout {
     int nodes, preds, ktab, total;           // byte offsets in a warp's shared memory (connections at 0)
 };
@@ -322,9 +347,9 @@ __global__ void __launch_bounds__(128) mutate_warp_kernel(const MutArgs a)
                     for (int i = lane; i < RN * N; i += 32) preds[i] = 0u;
                     __syncwarp();
                     for (int r = lane; r < N; r += 32)
-                        if (node_present(r)) insert32(ktab, kmask, kshift, (uint32_t)ns[5 * r] & 0xffffffu, (uint32_t)r);
+                        if (node_present(r)) insert_row(ktab, kmask, kshift, ns, (uint32_t)r);
                     __syncwarp();
-                    auto row_of = [&](float k) { return find32(ktab, kmask, kshift, (uint32_t)k & 0xffffffu); };
+                    auto row_of = [&](float k) { return find_row(ktab, kmask, kshift, ns, (uint32_t)k); };
                     for (int c = lane; c < C; c += 32) {
                         if (!conn_present(c)) continue;
                         const int x = row_of(cs[c].x), y = row_of(cs[c].y);
@@ -693,6 +718,7 @@ __host__ __device__ inline CrossWarpLayout cross_warp_layout(int N, int Np2, int
 
 __device__ __forceinline__ uint32_t pair_hash(uint32_t ki, uint32_t ko)
 {
+    // finalised with a multiplier of Wellons's hash prospector (2c1b3c6d)
     uint32_t h = ki * 0x9E3779B1u + ko * 0x85EBCA6Bu;
     h ^= h >> 15;
     h *= 0x2C1B3C6Du;
