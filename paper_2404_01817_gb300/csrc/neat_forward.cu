@@ -78,9 +78,12 @@ __global__ void __launch_bounds__(1024, 1) forward_kernel(const ForwardArgs a)
         pdl_wait();
         pdl_trigger();
     }
-    run_item<T1, PAIRS>(srec, v, bar, flags + gi, G, gi, lane, a.x + ((size_t)g * a.B + b0) * a.I,
-                        a.y + ((size_t)g * a.B + b0) * a.O, a.I, a.O, bt, a.tile, a.lg_split, a.val_floats, 0xffffffffu,
-                        &g_forward_error);
+    // a tile holds N rows: all columns at once (with the loop over columns of
+    // the plans' outgrown records around the walk, 8 and 40 vectors of 500 to
+    // 1024 rows took 4 to 11% longer)
+    run_item<T1, PAIRS, true>(srec, v, bar, flags + gi, G, gi, lane, a.x + ((size_t)g * a.B + b0) * a.I,
+                              a.y + ((size_t)g * a.B + b0) * a.O, a.I, a.O, bt, a.tile, a.lg_split, a.val_floats,
+                              0xffffffffu, &g_forward_error);
 }
 
 // One input vector per genome, one warp per genome, the record read where it

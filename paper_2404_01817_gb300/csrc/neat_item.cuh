@@ -507,7 +507,7 @@ __device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t b
     }
     if (h1.x > rec_limit) return false;
     const uint16_t *io = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.w);
-    if constexpr (!T1 && WHOLE) {
+    if constexpr (WHOLE) {
         if (((int)(h0.x & 0xffffu) << lgT) > vcap) return false;
     } else if constexpr (!T1)
         while (lgT > (PAIRS ? 1 : 0) && ((int)(h0.x & 0xffffu) << lgT) > vcap) --lgT;
