@@ -48,13 +48,6 @@ int allow_dynamic_smem(const void *kernel, size_t dynamic_bytes, const char *wha
     std::lock_guard<std::mutex> lk(g_smem_mu);
     auto it = g_smem_allowed.find({dev, kernel});
     if (it != g_smem_allowed.end() && it->second >= dynamic_bytes) return NEAT_OK;
-    if (it == g_smem_allowed.end()) {
-        // as much shared memory as an SM has: left to itself the driver gave
-        // some kernels room for four blocks where the SM holds six or eight
-        // (the lane programs' step: 3.45 instead of 3.57 ms per 1000 of them)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return cuda_fail(e, what);
-    }
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, kernel);
     if (e != cudaSuccess) return cuda_fail(e, what);
