@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(1024, 1) forward_kernel(const ForwardArgs a)
     // 1024 rows took 4 to 11% longer)
     run_item<T1, PAIRS, true>(srec, v, bar, flags + gi, G, gi, lane, a.x + ((size_t)g * a.B + b0) * a.I,
                               a.y + ((size_t)g * a.B + b0) * a.O, a.I, a.O, bt, a.tile, a.lg_split, a.val_floats,
-                              0xffffffffu, &g_forward_error);
+                              AlwaysFits{}, &g_forward_error);
 }
 
 // One input vector per genome, one warp per genome, the record read where it
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(32 * kDirectWarps) forward_direct_kernel(const
     float *v = reinterpret_cast<float *>(smem) + (size_t)gi * a.val_floats;
     if (lane == 0) flags[gi] = 0;
     run_item<true>(reinterpret_cast<const uint4 *>(a.rec + (size_t)g * a.stride), v, kNoBar, flags + gi, 32, gi, lane,
-                   a.x + (size_t)g * a.I, a.y + (size_t)g * a.O, a.I, a.O, 1, 1, 0, a.val_floats, 0xffffffffu,
+                   a.x + (size_t)g * a.I, a.y + (size_t)g * a.O, a.I, a.O, 1, 1, 0, a.val_floats, AlwaysFits{},
                    &g_forward_error);
 }
 

@@ -118,6 +118,7 @@ struct BucketDev {
     int rec_words;           // 16-byte words reserved for the record
     int rec_copy_bytes;
     int cta_begin, cta_items;
+    int spare;               // floats of the block's regions for an outgrown record's values
 };
 
 // A whole population as one bucket with the heuristic launch shape; gidx_dev

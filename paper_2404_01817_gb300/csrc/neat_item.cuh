@@ -463,6 +463,11 @@ __device__ __forceinline__ int ilog2(int x) { return 31 - __clz(x); }
 constexpr int kInputRegs = 8;   // inputs prefetched into registers per thread
 constexpr uint32_t kNoBar = 0xffffffffu;
 
+// Records and nodes of the sizes that the shapes were made for.
+struct AlwaysFits {
+    __device__ __forceinline__ bool operator()(uint32_t, int) const { return true; }
+};
+
 // Everything of one work item after its record copy was issued by lane 0
 // (mbarrier `bar` initialised and armed, `flag` set to 0, both before the
 // call; bar kNoBar: the record is read where it is, nothing to wait for): inputs
@@ -472,15 +477,15 @@ constexpr uint32_t kNoBar = 0xffffffffu;
 // tile, walks the levels and writes the outputs.
 //   xb: inputs of the item [bt][I]; yb: its outputs [bt][O]; vcap: floats of
 //   the value tile, at least one column of the genome's nodes (a genome with
-//   more nodes than the tile has rows takes fewer columns at a time).
-// False, with nothing evaluated, when the record is longer than rec_limit
-// bytes (the part that was copied), or (WHOLE: all columns at once) has more
-// nodes than the tile has rows.  PAIRS: two columns per thread (tile at
-// least 2, at most 2 G; vcap at least two columns).
-template <bool T1, bool PAIRS = false, bool WHOLE = false>
+//   more nodes than the tile has rows takes fewer columns at a time; WHOLE: it
+//   has the rows, all columns at once).
+//   fits(bytes of the record, values of its columns): asked once the record is
+//   there; where it is false, run_item returns false with nothing evaluated.
+// PAIRS: two columns per thread (tile 64, WHOLE).
+template <bool T1, bool PAIRS = false, bool WHOLE = false, typename Fits>
 __device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t bar, volatile int *flag, int G,
                                          int gi, int lane, const float *__restrict__ xb, float *__restrict__ yb,
-                                         int I, int O, int bt, int tile, int lg_split, int vcap, uint32_t rec_limit,
+                                         int I, int O, int bt, int tile, int lg_split, int vcap, const Fits &fits,
                                          unsigned int *err)
 {
     int lgT = T1 ? 0 : ilog2(tile);
@@ -505,12 +510,10 @@ __device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t b
         for (int i = lane; i < bt * O; i += G) yb[i] = __int_as_float(0x7fc00000);
         return true;
     }
-    if (h1.x > rec_limit) return false;
+    if (!fits(h1.x, (int)(h0.x & 0xffffu) << lgT)) return false;
     const uint16_t *io = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.w);
-    if constexpr (WHOLE) {
-        if (((int)(h0.x & 0xffffu) << lgT) > vcap) return false;
-    } else if constexpr (!T1)
-        while (lgT > (PAIRS ? 1 : 0) && ((int)(h0.x & 0xffffu) << lgT) > vcap) --lgT;
+    if constexpr (!T1 && !WHOLE)
+        while (lgT > 0 && ((int)(h0.x & 0xffffu) << lgT) > vcap) --lgT;
     const int step = T1 ? 1 : 1 << lgT;
     constexpr bool kOnce = T1 || WHOLE;
     for (int c0 = 0; c0 < (kOnce ? 1 : bt); c0 += step) {   // once, unless the nodes outgrow the tile's rows

@@ -233,14 +233,60 @@ compact_kernel(const CompactPop *__restrict__ pops, int np, const CompactPop one
     }
 }
 
-// An item whose record or nodes outgrow its group's region (a record changed
-// since the plan chose its shapes): read where it lies.
-template <bool T1>
-__device__ __noinline__ void run_item_in_place(const uint4 *rec, float *v, volatile int *flag, int G, int gi, int lane,
-                                               const float *xb, float *yb, int I, int O, int bt, int tile, int lg_split,
-                                               int vcap, unsigned int *err)
+// The items of a block item whose record or nodes outgrow their group's region
+// (records changed since the plan chose its shapes): one after the other, the
+// record read where it lies, the values in the memory of all regions, which
+// holds a column of any genome of the population (`spare` floats).  So a region
+// is no larger than its bucket's genomes need: with room for max_nodes values
+// in every group, 4000 genomes of 14 nodes in 1024 rows and 64 vectors took
+// 16.4 us a step instead of 15.3.  Every thread of the block calls it.
+__device__ __noinline__ void run_outgrown(const BucketDev &d, int ci, int step, bool late, float *v, int *flags,
+                                          unsigned int *err)
 {
-    run_item<T1>(rec, v, kNoBar, flag, G, gi, lane, xb, yb, I, O, bt, tile, lg_split, vcap, 0xffffffffu, err);
+    const int G = d.G, gi = threadIdx.x >> d.lgG, lane = threadIdx.x & (G - 1);
+    const long item = (long)(ci - d.cta_begin) * d.gpc + gi;
+    const int k = late ? (int)(item / d.tiles) : 0, g = __ldg(d.gidx + k);
+    const int b0 = (int)(item - (long)k * d.tiles) * d.tile;
+    const uint4 *rec = reinterpret_cast<const uint4 *>(d.rec + (size_t)g * d.stride);
+    const float *xb = d.x + d.x_step * step + ((size_t)g * d.B + b0) * d.I;
+    float *yb = d.y + d.y_step * step + ((size_t)g * d.B + b0) * d.O;
+    for (int turn = 0; turn < d.gpc; ++turn) {
+        if (late && turn == gi) {
+            if (d.tile == 1)
+                run_item<true>(rec, v, kNoBar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split, d.spare,
+                               AlwaysFits{}, err);
+            else
+                run_item<false>(rec, v, kNoBar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, min(d.tile, d.B - b0), d.tile, 0,
+                                d.spare, AlwaysFits{}, err);
+        }
+        __syncthreads();
+    }
+}
+
+// A work item whose record's copy is on its way; false, with nothing evaluated,
+// when the record or its nodes outgrow the group's region.  The walk of one
+// vector is a function of its own: beside the tiles' in one body its loop came
+// out slower (a launch of one vector each, 231 genomes of 26 and of 77 rows 18.5
+// us, 14.5 as a function; the tiles' as a function too: 8 to 31 vectors 3 to 8%
+// slower).
+template <bool T1>
+__device__ __forceinline__ bool staged_item(const BucketDev &d, uint4 *srec, uint32_t bar, int *flag, int gi, int lane,
+                                            int g, int b0, int step)
+{
+    const float *xb = d.x + d.x_step * step + ((size_t)g * d.B + b0) * d.I;
+    float *yb = d.y + d.y_step * step + ((size_t)g * d.B + b0) * d.O;
+    const auto fits = [&](uint32_t bytes, int values) {
+        return bytes <= (uint32_t)d.rec_words * 16u && values <= (d.region_words - d.rec_words) * 4;
+    };
+    return run_item<T1, false, true>(srec, reinterpret_cast<float *>(srec + d.rec_words), bar, flag, d.G, gi, lane, xb, yb,
+                                     d.I, d.O, T1 ? 1 : min(d.tile, d.B - b0), T1 ? 1 : d.tile, T1 ? d.lg_split : 0, 0, fits,
+                                     &g_plan_error);
+}
+
+__device__ __noinline__ bool staged_vector(const BucketDev &d, uint4 *srec, uint32_t bar, int *flag, int gi, int lane,
+                                           int g, int b0, int step)
+{
+    return staged_item<true>(d, srec, bar, flag, gi, lane, g, b0, step);
 }
 
 template <bool PDL>
@@ -248,12 +294,13 @@ __global__ void __launch_bounds__(1024, 1)
 plan_kernel(const BucketDev *__restrict__ buckets, int nb, int item_lo, int item_hi, unsigned int *counter, int step)
 {
     extern __shared__ __align__(16) uint4 smem[];
-    __shared__ int s_ci;
+    __shared__ int s_ci, s_late;
     const int NT = blockDim.x;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
     int *flags = reinterpret_cast<int *>(bars + NT);
     uint4 *regions = smem + forward_header_words(NT);
     bool waited = !PDL;
+    if (threadIdx.x == 0) s_late = 0;
     for (;;) {
         if (threadIdx.x == 0) s_ci = item_lo + (int)atomicAdd(counter, 1u);
         __syncthreads();
@@ -273,7 +320,7 @@ plan_kernel(const BucketDev *__restrict__ buckets, int nb, int item_lo, int item
         uint4 *srec = regions + (size_t)gi * d.region_words;
         const uint32_t bar = smem_addr(bars + gi);
         int g = 0, b0 = 0;
-        bool staged = true;
+        bool staged = active;
         if (active) {
             const int k = (int)(item / d.tiles);
             g = __ldg(d.gidx + k);
@@ -299,32 +346,17 @@ plan_kernel(const BucketDev *__restrict__ buckets, int nb, int item_lo, int item
             pdl_trigger();
             waited = true;
         }
-        if (active) {
-            const int bt = min(d.tile, d.B - b0);
-            const float *xb = d.x + d.x_step * step + ((size_t)g * d.B + b0) * d.I;
-            float *yb = d.y + d.y_step * step + ((size_t)g * d.B + b0) * d.O;
-            float *v = reinterpret_cast<float *>(srec + d.rec_words);
-            const int vcap = (d.region_words - d.rec_words) * 4;
-            const uint32_t limit = (uint32_t)d.rec_words * 16u;
-            const bool t1 = d.tile == 1;
-            bool done = false;
-            if (staged)
-                done = t1 ? run_item<true, false, true>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split,
-                                           vcap, limit, &g_plan_error)
-                          : run_item<false, false, true>(srec, v, bar, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, vcap,
-                                            limit, &g_plan_error);
-            if (!done) {
-                const uint4 *grec = reinterpret_cast<const uint4 *>(d.rec + (size_t)g * d.stride);
-                if (t1)
-                    run_item_in_place<true>(grec, v, flags + gi, G, gi, lane, xb, yb, d.I, d.O, 1, 1, d.lg_split, vcap,
-                                            &g_plan_error);
-                else
-                    run_item_in_place<false>(grec, v, flags + gi, G, gi, lane, xb, yb, d.I, d.O, bt, d.tile, 0, vcap,
-                                             &g_plan_error);
-            }
-        }
+        bool late = active && !staged;
+        if (staged)
+            late = !(d.tile == 1 ? staged_vector(d, srec, bar, flags + gi, gi, lane, g, b0, step)
+                                 : staged_item<false>(d, srec, bar, flags + gi, gi, lane, g, b0, step));
+        if (late) s_late = 1;
         __syncthreads();
-        if (active && staged && lane == 0) mbar_inval(bar);   // re-initialised by the next item using this slot
+        if (staged && lane == 0) mbar_inval(bar);      // re-initialised by the next item using this slot
+        if (s_late) {                                  // the same for all: cleared behind run_outgrown's barriers
+            run_outgrown(d, ci, step, late, reinterpret_cast<float *>(regions), flags, &g_plan_error);
+            if (threadIdx.x == 0) s_late = 0;
+        }
     }
 }
 
@@ -356,6 +388,10 @@ bool shape_ok(const Shape &s, int NT)
     const auto p2 = [](int x) { return x > 0 && (x & (x - 1)) == 0; };
     return p2(s.G) && s.G <= NT && p2(s.tile) && s.tile <= s.G && (s.split == 1 || s.split == 2 || s.split == 4);
 }
+
+// Floats of a block's regions (a multiple of 16 bytes), at least a column of the
+// population's largest genome (run_outgrown).
+int spare_floats(size_t regions, int max_nodes) { return std::max((int)(regions / 4), (max_nodes + 3) & ~3); }
 
 // Launch shape without timing: as neat_default_launch, with groups of at
 // most NT threads (the persistent block).
@@ -410,13 +446,10 @@ struct neat_plan {
 namespace neat {
 namespace {
 
-size_t region_bytes(const neat_plan *P, const HostBucket &b)
+size_t region_bytes(const HostBucket &b)
 {
     const size_t rec = (size_t)align16((uint32_t)b.max_used);
-    // one column of any genome of the population fits, whatever its record
-    // becomes (run_item takes fewer columns at a time then)
-    const int vals = std::max(b.max_rows * b.shape.tile, P->pops[b.pop_index].dims.max_nodes);
-    return (rec + 4u * (size_t)((vals + 3) & ~3) + 15) & ~(size_t)15;
+    return (rec + 4u * (size_t)((b.max_rows * b.shape.tile + 3) & ~3) + 15) & ~(size_t)15;
 }
 
 // Compact records from the records as they are now, and `counters` cleared.
@@ -475,7 +508,7 @@ int layout(neat_plan *P, cudaStream_t s)
         if (!shape_ok(h.shape, NT)) return invalid("plan: invalid bucket launch shape");
         d.G = h.shape.G;
         d.lgG = lg(d.G);
-        const size_t reg = region_bytes(P, h);
+        const size_t reg = region_bytes(h);
         int gpc = NT / d.G;
         if (d.G > 32) gpc = std::min(gpc, 15);
         while (gpc > 1 && reg * gpc > 200u * 1024u) --gpc;
@@ -489,7 +522,8 @@ int layout(neat_plan *P, cudaStream_t s)
         d.cta_begin = cta;
         d.cta_items = (int)((items + gpc - 1) / gpc);
         cta += d.cta_items;
-        smem_regions = std::max(smem_regions, reg * gpc);
+        d.spare = spare_floats(reg * gpc, pd.dims.max_nodes);
+        smem_regions = std::max(smem_regions, 4u * (size_t)d.spare);
         bd.push_back(d);
     }
     P->bd = bd;
@@ -499,7 +533,7 @@ int layout(neat_plan *P, cudaStream_t s)
     {
         size_t best = 0;
         for (size_t i = 0; i < bd.size(); ++i) {
-            const size_t f = (size_t)bd[i].region_words * 16 * bd[i].gpc;
+            const size_t f = 4u * (size_t)bd[i].spare;
             if (f > best) {
                 best = f;
                 P->max_footprint_bucket = order[i];
@@ -573,7 +607,7 @@ int launch_step(neat_plan *P, int lo, int hi, unsigned int *ctr, int step, bool 
 float time_bucket(neat_plan *P, int bi, cudaStream_t s, int reps)
 {
     const BucketDev &d = P->bd[bi];
-    P->smem_override = (size_t)d.region_words * 16 * d.gpc + 16u * forward_header_words(P->block_threads);
+    P->smem_override = 4u * (size_t)d.spare + 16u * forward_header_words(P->block_threads);
     const int grid_saved = P->grid;
     {
         int dev = 0, sms = 152, smem_sm = 233472;
@@ -655,7 +689,7 @@ size_t footprint(const neat_plan *P, const HostBucket &h)
 {
     int gpc = P->block_threads / h.shape.G;
     if (h.shape.G > 32) gpc = std::min(gpc, 15);
-    return region_bytes(P, h) * gpc;
+    return region_bytes(h) * gpc;
 }
 
 int autotune(neat_plan *P, cudaStream_t s, float *step_ms)
@@ -1254,7 +1288,8 @@ extern "C" int neat_forward_multi_noalloc(const neat_pop_desc *pops, int32_t npo
         d.cta_begin = (int)cta;
         d.cta_items = (int)items;
         cta += items;
-        smem_regions = std::max(smem_regions, reg * gpc);
+        d.spare = spare_floats(reg * gpc, pd.dims.max_nodes);
+        smem_regions = std::max(smem_regions, 4u * (size_t)d.spare);
     }
     if (nb == 0) return NEAT_OK;
     const size_t smem = smem_regions + 16u * forward_header_words(NT);
@@ -1339,7 +1374,8 @@ int fill_population_bucket(const neat_pop_desc &pd, const int32_t *gidx_dev, int
     d.rec_copy_bytes = own_size ? 0 : (int)rec;
     d.cta_begin = cta_begin;
     d.cta_items = (int)(((long)d.n_genomes * d.tiles + gpc - 1) / gpc);
-    *footprint = reg * gpc;
+    d.spare = spare_floats(reg * gpc, pd.dims.max_nodes);
+    *footprint = 4u * (size_t)d.spare;
     return NEAT_OK;
 }
 
