@@ -297,6 +297,19 @@ cudaEvent_t take_event(neat_server *S)
     return e;
 }
 
+// Whether a request's steps are worth the compact copies, which cost it 13 to 25
+// us (a launch that its first step waits for).  What a step of it saves alone on
+// the device, measured at 500 to 1000 genomes of 16 to 1000 rows: up to 16 vectors
+// at most some 5 us, and less the fewer node rows there are to walk; beyond, in
+// proportion to the rows times the tiles of 32, once these fill the device.
+bool copies_pay(const neat_request &r)
+{
+    const double rows = (double)r.pop * r.dims.max_nodes;
+    const double step_us = r.batch <= 16 ? std::min(5.0, rows / 10000.0)
+                                         : (rows * ((r.batch + 31) / 32) - 80000.0) / 16000.0;
+    return r.steps * step_us >= 20.0;
+}
+
 // After the transform: copies of the records without the nodes that no output
 // depends on, evaluated from then on.  They take the place of the genome
 // tensors, where these are large enough; how large the copies are comes back
@@ -307,7 +320,7 @@ int compact_request(neat_server *S, Request *R)
     const neat_request &r = R->r;
     unsigned char *base = S->pool + R->off;
     const size_t bytes = record_stride(r.dims) * (size_t)r.pop;
-    if (R->o_nodes != 0 || bytes > R->o_rec) return NEAT_OK;
+    if (!copies_pay(r) || R->o_nodes != 0 || bytes > R->o_rec) return NEAT_OK;
     uint32_t *largest = reinterpret_cast<uint32_t *>(base + R->o_status);      // the status words are not needed
     cudaError_t e = cudaMemsetAsync(largest, 0, 8, S->stream);
     if (e != cudaSuccess) return cuda_fail(e, "serve: clear sizes");
