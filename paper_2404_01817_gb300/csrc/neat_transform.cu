@@ -454,18 +454,24 @@ __global__ void __launch_bounds__(128) transform_warp_kernel(const TransformArgs
 //      end by their keys, in a pass of their own where there are any); an edge
 //      takes the next free place among its destination's edges, in whatever
 //      order they arrive, and the next place of a list of all edges;
-////   3. layered Kahn: one pass over the active edges per level;
+//   3. layered Kahn: one pass over the active edges per level;
 //   4. positions = rank of (level, row): every 32 rows count their levels,
 //      the counts are summed over the rows before;
 //   5. edges in (destination position, connection row) order: every edge
 //      counts the edges of its destination with a lower row (a node has a few
-//      edges; one with 1000 costs 1000 reads per edge, all edges at once);
+//      edges); the rows of a destination with more than kHubEdges are sorted
+//      first, by a warp through a bit per connection row, and searched;
 //      the record staged in shared memory and written in one coalesced pass.
 // Bound by issue and barriers (57% of the issue slots at 30 warps per SM).
 // 4096 genomes of 500 / 2000 rows: 172 us in blocks of 256 threads (four per
 // SM by 48 KB of shared memory each), against 411 us for the form whose one
 // warp placed all edges in chunks of 32, waiting for each chunk's weights, and
-// 253 us for that placement spread over 16 warps with match-based ranks.
+// 253 us for that placement spread over 16 warps with match-based ranks.  608
+// genomes of 1000 inputs, each feeding 8 outputs: 165 us (768 where every edge
+// counts through its output's 1000; that warp 497); 2000 of 500 inputs and 4
+// outputs 111 (347; 652).
+constexpr int kHubEdges = 128;   // above 128 node rows the bits of one destination always fit two words per row
+
 struct BlockLayout {
     size_t ktab, ptab, edge_of, ints, list, rows, io, total;
     int level, indeg, cnt, place, tot;       // offsets in `ints` (words)
@@ -550,6 +556,32 @@ __device__ __noinline__ bool duplicate_dangling_block(const float4 *cn, int C, c
     return dup;
 }
 
+// The connection rows list[0 .. m) in ascending order, by one warp; bits: a word
+// for every 32 of the C connection rows.  (As a function of its own, or the search
+// too: the call alone cost genomes without such a destination 1 to 5%.)
+__device__ __forceinline__ void sort_rows(uint16_t *list, int m, uint32_t *bits, int C, int lane)
+{
+    const int words = (C + 31) >> 5;
+    for (int i = lane; i < words; i += 32) bits[i] = 0u;
+    __syncwarp();
+    for (int i = lane; i < m; i += 32) atomicOr(bits + (list[i] >> 5), 1u << (list[i] & 31u));
+    __syncwarp();
+    int carry = 0;
+    for (int base = 0; base < words; base += 32) {
+        const uint32_t mine = base + lane < words ? bits[base + lane] : 0u;
+        int incl = __popc(mine);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        int at = carry + incl - __popc(mine);
+        for (uint32_t b = mine; b; b &= b - 1u) list[at++] = (uint16_t)(32 * (base + lane) + __ffs(b) - 1);
+        carry += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    __syncwarp();
+}
+
 __global__ void __launch_bounds__(512, 2) transform_block_kernel(const TransformArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -575,8 +607,9 @@ __global__ void __launch_bounds__(512, 2) transform_block_kernel(const Transform
     uint16_t *io_row = reinterpret_cast<uint16_t *>(sm + lay.io);
 
     __shared__ unsigned int st, acts_seen, aggs_seen, lead_inputs;
-    __shared__ int n_present, n_edges, max_level;
+    __shared__ int n_present, n_edges, max_level, hubs;
     if (tid == 0) {
+        hubs = 0;
         st = 0;
         acts_seen = 0;
         aggs_seen = 0;
@@ -785,6 +818,7 @@ __global__ void __launch_bounds__(512, 2) transform_block_kernel(const Transform
         const bool input = key < (float)I;
         const uint32_t act = input ? (uint32_t)kInputAct : (uint32_t)__ldg(nd + r * 5 + 4);
         if (!input) lead = min(lead, (unsigned)p);                           // leading positions that are inputs
+        if (cnt[r] > kHubEdges) hubs = 1;
         nodes_st[p] = make_uint4(__float_as_uint(bias), __float_as_uint(resp),
                                  (uint32_t)first | ((uint32_t)cnt[r] << 16), act | (agg << 8) | ((uint32_t)r << 16));
     }
@@ -796,6 +830,22 @@ __global__ void __launch_bounds__(512, 2) transform_block_kernel(const Transform
         list[(uint32_t)(place[(e >> 10) & 1023u] >> 16) + (e >> 20)] = rows_of[k];
     }
     __syncthreads();
+    if (hubs) {
+        // the levels and positions by row have been used: their memory holds the bits
+        const int words = (C + 31) >> 5, sorters = min(nw, 2 * N / words);
+        if (warp < sorters) {
+            int seen = 0;
+            for (int base = 0; base < N; base += 32) {
+                unsigned m = __ballot_sync(all, base + lane < N && cnt[base + lane] > kHubEdges);
+                for (; m; m &= m - 1u) {
+                    const int d = base + __ffs(m) - 1;
+                    if (seen++ % sorters == warp)
+                        sort_rows(list + (place[d] >> 16), cnt[d], reinterpret_cast<uint32_t *>(ints) + warp * words, C, lane);
+                }
+            }
+        }
+        __syncthreads();
+    }
     uint2 *edges_st = reinterpret_cast<uint2 *>(ptab);
     for (int k = tid; k < E; k += nt) {
         const uint32_t e = edge_of[k];
@@ -804,7 +854,14 @@ __global__ void __launch_bounds__(512, 2) transform_block_kernel(const Transform
         const int d = (int)((e >> 10) & 1023u);
         const int first = place[d] >> 16, m = cnt[d];
         int rank = 0;
-        for (int i = 0; i < m; ++i) rank += (int)list[first + i] < c ? 1 : 0;
+        if (m > kHubEdges) {
+            for (int above = m; rank + 1 < above;) {                         // list[first + rank] <= c < list[first + above]
+                const int mid = (rank + above) >> 1;
+                if ((int)list[first + mid] <= c) rank = mid; else above = mid;
+            }
+        } else {
+            for (int i = 0; i < m; ++i) rank += (int)list[first + i] < c ? 1 : 0;
+        }
         edges_st[first + rank] = make_uint2(__float_as_uint(w), (uint32_t)place[e & 1023u] & 0xffffu);
     }
     uint16_t *io_out = reinterpret_cast<uint16_t *>(rec + o.io);
