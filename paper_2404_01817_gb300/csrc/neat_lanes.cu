@@ -1235,10 +1235,16 @@ int make_lanes_args(const void *lanes, int32_t pop, const neat_dims &d, const fl
 // Four: up to 2.5 blocks per SM, and where no more than four fit on one.  With
 // more blocks a full SM is busy with fewer warps each, and two are as good or
 // better: 9 500 genomes of 40 nodes 13.3, 12.8, 14.2; 10 000 of 24 nodes 9.4,
-// 8.7, 9.1; of 48 nodes 15.8, 14.4, 14.8.  One, where more than four blocks per
-// SM are launched and an SM has room for a part of the next launch's share:
-// overlapping launches then spread over the SMs unevenly, which costs most
-// when a block keeps its SM busy (10 000 of 32 nodes 12.0, 12.8, 15.0).
+// 8.7, 9.1; of 48 nodes 15.8, 14.4, 14.8.  One: from six blocks per SM and
+// launch on, where an SM has room for six or more, they fill it by themselves
+// (one, two, four, with overlapping launches: 16 000 genomes of 24 nodes 11.5,
+// 14.0, 14.7; of 32 12.8, 14.3, 17.4; of 40 16.1, 17.1, 18.1; 14 500 of 16 nodes
+// 7.6, 8.3, 11.7; where fewer fit, 16 000 of 48 nodes 19.5, 19.4, 20.1, of 64
+// 24.8, 22.9, 22.9; launches that do not overlap gain less or lose up to 5%: 13
+// 000 of 32 nodes 12.2, 11.6, 12.6); and at five where an SM has room for a part
+// of the next launch's share, seven or eight, so that overlapping launches spread
+// over the SMs unevenly (11 000 of 32 nodes 11.9, 12.9, 15.3; with room for six,
+// 11 000 of 40 nodes 13.4, 13.1, 14.3, or ten, 11 000 of 24 nodes 9.2, 8.7, 12.7).
 int rnn_warps(int programs, size_t smem)
 {
     int dev = 0, sms = 152, smem_sm = 228 * 1024;
@@ -1249,7 +1255,8 @@ int rnn_warps(int programs, size_t smem)
     const long fit = smem_sm / (long)(smem + 1024u);   // 1 KB reserved per block
     if (2L * programs <= 5L * sms || fit <= 4) return 4;
     const long need = (programs + sms - 1L) / sms;
-    return need > 4 && fit > need + 1 && fit < 2 * need - 1 ? 1 : 2;
+    if (need == 5) return fit == 7 || fit == 8 ? 1 : 2;
+    return need >= 6 && fit >= 6 ? 1 : 2;
 }
 
 int launch_lanes_rnn(const LanesArgs &a, int warps, int K, bool pdl, cudaStream_t s)
