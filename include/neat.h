@@ -196,9 +196,9 @@ NEAT_API int neat_transform(const float *nodes_dev, const float *conns_dev, int3
  *   inputs_dev       f32 [pop][batch][I]
  *   outputs_dev      f32 [pop][batch][O] (written; NaN for genomes with an error bit)
  * The launch shape is chosen from (pop, dims, batch), as neat_default_launch
- * says; 33 to 64 vectors for many large genomes are evaluated two per thread
- * where the genomes' values are small enough, and one vector for many large genomes reads
- * the records where they lie.  The results do not depend on it.
+ * says; 33 to 64 vectors of genomes of 64 to 255 node rows are evaluated two per
+ * thread where there are genomes enough to fill the device, and one vector for many
+ * large genomes reads the records where they lie.  The results do not depend on it.
  * Errors: NEAT_EINVAL, NEAT_ECUDA.
  */
 NEAT_API int neat_forward(const void *transformed_dev, int32_t pop, neat_dims d,

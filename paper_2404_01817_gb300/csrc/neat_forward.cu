@@ -345,7 +345,7 @@ DeviceCaps device_caps()
 
 // Groups per block: all items resident in as few waves as possible, with the
 // items spread evenly over the SMs (fewest groups on the busiest SM).
-int choose_groups_per_block(long items, int group, size_t per_group, const DeviceCaps &caps)
+int choose_groups_per_block(long items, int group, size_t per_group, const DeviceCaps &caps, long *waves_out = nullptr)
 {
     const int max_gpb = group > 32 ? std::min(15, 1024 / group) : 1024 / group;
     int best = 1;
@@ -379,6 +379,7 @@ int choose_groups_per_block(long items, int group, size_t per_group, const Devic
             best_load = load;
         }
     }
+    if (waves_out) *waves_out = best_waves;
     return best;
 }
 
@@ -386,10 +387,44 @@ int choose_groups_per_block(long items, int group, size_t per_group, const Devic
 }  // namespace neat
 
 namespace neat {
-int groups_per_block_for(long items, int group, size_t per_group)
+int groups_per_block_for(long items, int group, size_t per_group, long *waves)
 {
-    return choose_groups_per_block(items, group, per_group, device_caps());
+    return choose_groups_per_block(items, group, per_group, device_caps(), waves);
 }
+
+namespace {
+
+// The launch of two columns per thread in one tile of 64, for 33 to 64 vectors,
+// where it is the faster one.  It walks a genome once, by half the threads of the
+// two tiles of 32 that would, so it needs the SMs full: tiles of 32 must put 20
+// warps on each.  Sixteen or fewer, any rows: 10 to 20% slower; 20 to 28: up to
+// 1.3 times as fast.  Then, by the threads of a tile row (tile_row_threads):
+//   four (128 to 255 rows): always (400 genomes 1.03 to 1.2, 3300 1.25 to 1.6);
+//   two (64 to 127): while all genomes fit the SMs at once, 1.1 to 1.3 (760 to
+//     1064 genomes of 100 rows), and again from 50 warps on, 1.02 to 1.8; in
+//     between it is 0.85 to 1.3, as the tiles of 32 happen to divide;
+//   one, or eight and more: 40 and 56 rows 0.8 to 0.9, 256 and 320 1.0: never.
+// Beyond 75 KB a group fewer than three share an SM.  (Ratios of launches, 15
+// sizes of 40 to 320 rows with four connections each, 150 to 3300 genomes, 33, 48
+// and 64 vectors alike.)
+constexpr size_t kMaxPairGroupSmem = 75u * 1024u;
+
+bool pairs_launch(int pop, const neat_dims &d, size_t rec_bytes, const DeviceCaps &caps, neat_launch *L)
+{
+    const int rows = tile_row_threads(d.max_nodes);
+    if (rows != 2 && rows != 4) return false;
+    const long warps = (2L * pop + caps.sms - 1) / caps.sms * rows;
+    if (warps < 20) return false;
+    const size_t per_group = rec_bytes + 4u * 64u * (size_t)d.max_nodes;
+    if (per_group > kMaxPairGroupSmem) return false;
+    long waves = 0;
+    L->tile = 64;
+    L->group = 32 * rows;
+    L->groups_per_block = groups_per_block_for(pop, L->group, per_group, &waves);
+    return rows == 4 || waves == 1 || warps >= 50;
+}
+
+}  // namespace
 }  // namespace neat
 
 extern "C" int neat_default_launch(int32_t pop, neat_dims d, int32_t batch, neat_launch *out)
@@ -455,28 +490,16 @@ extern "C" int neat_forward_ex(const void *transformed_dev, int32_t pop, neat_di
         const cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? NEAT_OK : cuda_fail(e, "forward: launch");
     }
-    if (!launch_host && batch > 32 && batch <= 64 && d.max_nodes >= kMinPairNodes && pop >= kMinPairPop) {
-        // two columns per thread in tiles of 64, where four such groups fit an
-        // SM, there are genomes enough to fill it and a level has nodes enough
-        // for the fewer threads (a launch, 40 vectors, sum and tanh: 1200
-        // genomes of 50 rows 17 us in tiles of 32 and 19 in pairs, 300 of 101
-        // rows 18 and 19, 2400 of 101 rows 51 and 45; 67 vectors, whose second
-        // tile is nearly empty: 73 and 95).  1001 genomes of 101 / 403 rows and
-        // 37 vectors, mixed activations and aggregations: 51 -> 46 us with the
-        // transform (one tile of 37 instead of tiles of 32 and 5).  (In the
-        // plan's kernel, whose registers it overran, the same shapes took 195
-        // instead of 189 us a step)
+    // (In the plan's kernel, whose registers the pairs overran, the same shapes
+    // took 195 instead of 189 us a step)
+    if (!launch_host && batch > 32 && batch <= 64) {
         neat_launch W = L;
-        W.tile = 64;
-        W.group = 32 * tile_row_threads(d.max_nodes);
-        const size_t per_group = (size_t)a.rec_words * 16 + 4u * 64u * (size_t)d.max_nodes;
-        if (per_group <= kMaxPairGroupSmem) {
+        if (pairs_launch(pop, d, (size_t)a.rec_words * 16, device_caps(), &W)) {
             a.pairs = 1;
             a.tile = W.tile;
             a.group = W.group;
-            a.tiles = (batch + W.tile - 1) / W.tile;
+            a.tiles = 1;
             a.val_floats = a.N * W.tile;
-            W.groups_per_block = groups_per_block_for((long)pop * a.tiles, W.group, per_group);
             return launch_forward(a, W, as_stream(stream));
         }
     }

@@ -57,11 +57,6 @@ int allow_dynamic_smem(const void *kernel, size_t dynamic_bytes, const char *wha
 // Shared memory one group's record and value tiles may take in a default
 // launch shape (room left for the block's barriers).
 constexpr size_t kMaxGroupSmem = 200u * 1024u;
-// The same for a tile of 64 columns, two per thread: beyond, fewer than four
-// groups share an SM and the tile of 32 is the better one.
-constexpr size_t kMaxPairGroupSmem = 48u * 1024u;
-constexpr int kMinPairNodes = 96, kMinPairPop = 1000;
-
 // Threads per tile row for a genome of up to n nodes and a batch of several
 // input vectors: about one per 32 nodes (a level of a large genome holds
 // tens of nodes), a power of two in 1..16.
@@ -87,7 +82,7 @@ struct ForwardArgs {
     int val_floats;          // floats of shared memory for node values (N * tile, rounded to 4)
     int rec_copy_bytes;      // bytes of each record copied in one piece (0: read the size from its header)
     const int32_t *order;    // genome of work item k / tiles (NULL: identity)
-    int pairs;               // two columns per thread (tile at most 2 x group)
+    int pairs;               // two columns per thread (tile 64, group a multiple of 32)
 };
 
 // 16-byte words before the groups' regions in a forward block's shared
@@ -146,7 +141,7 @@ int read_substrate_error(unsigned int *v, int clear);  // neat_substrate.cu
 int read_lanes_error(unsigned int *v, int clear);      // neat_lanes.cu
 // Groups per block that put `items` groups of `group` threads, each needing
 // `per_group` bytes of shared memory, in the fewest waves with the busiest SM
-// least loaded (neat_forward.cu).
-int groups_per_block_for(long items, int group, size_t per_group);
+// least loaded (neat_forward.cu); *waves (may be NULL): how many.
+int groups_per_block_for(long items, int group, size_t per_group, long *waves = nullptr);
 
 }  // namespace neat

@@ -237,26 +237,27 @@ __device__ __forceinline__ void walk_tile(const uint4 *nodes, const uint2 *edges
 
 // ---- two adjacent columns per thread
 //
-// A row of T columns is evaluated by T / 2 threads, columns 2 l and 2 l + 1 in
+// A tile row of 64 columns is evaluated by 32 threads, columns 2 l and 2 l + 1 in
 // thread l: the node's entry, its dispatches and its edges are read once for
 // both, their values are one 8-byte read and their sums run as a packed pair.
 // Each column's operations are those of eval_node_tile in the same order, so
 // the bits are too.
+constexpr int kLgPairTile = 6;
+
 template <int EC>
-__device__ __forceinline__ f2 sum_edges_pair(const uint2 *__restrict__ e, const char *__restrict__ v, int lgT)
+__device__ __forceinline__ f2 sum_edges_pair(const uint2 *__restrict__ e, const char *__restrict__ v)
 {
     f2 q[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
     for (int i = 0; i < EC; ++i) {
         const uint2 t = e[i];
-        const f2 x = *reinterpret_cast<const f2 *>(v + ((size_t)t.y << (lgT + 2)));
+        const f2 x = *reinterpret_cast<const f2 *>(v + (t.y << (kLgPairTile + 2)));
         q[i & 3] = fma2(pack2(__uint_as_float(t.x), __uint_as_float(t.x)), x, q[i & 3]);
     }
     return add2(add2(q[0], q[1]), add2(q[2], q[3]));
 }
 
-__device__ __forceinline__ f2 sum_edges_pair_any(const uint2 *__restrict__ e, uint32_t ec, const char *__restrict__ v,
-                                                 int lgT)
+__device__ __forceinline__ f2 sum_edges_pair_any(const uint2 *__restrict__ e, uint32_t ec, const char *__restrict__ v)
 {
     f2 q[4] = {0ull, 0ull, 0ull, 0ull};
     for (uint32_t i = 0; i < ec; i += 4) {
@@ -264,7 +265,7 @@ __device__ __forceinline__ f2 sum_edges_pair_any(const uint2 *__restrict__ e, ui
         for (int k = 0; k < 4; ++k) {
             if (i + k < ec) {
                 const uint2 t = e[i + k];
-                const f2 x = *reinterpret_cast<const f2 *>(v + ((size_t)t.y << (lgT + 2)));
+                const f2 x = *reinterpret_cast<const f2 *>(v + (t.y << (kLgPairTile + 2)));
                 q[k] = fma2(pack2(__uint_as_float(t.x), __uint_as_float(t.x)), x, q[k]);
             }
         }
@@ -273,8 +274,7 @@ __device__ __forceinline__ f2 sum_edges_pair_any(const uint2 *__restrict__ e, ui
 }
 
 template <uint32_t AGG>
-__device__ __forceinline__ float2 fold_edges_pair(const uint2 *__restrict__ e, uint32_t ec, const char *__restrict__ v,
-                                                  int lgT)
+__device__ __forceinline__ float2 fold_edges_pair(const uint2 *__restrict__ e, uint32_t ec, const char *__restrict__ v)
 {
     float q[4][2];
 #pragma unroll
@@ -284,7 +284,7 @@ __device__ __forceinline__ float2 fold_edges_pair(const uint2 *__restrict__ e, u
         for (int k = 0; k < 4; ++k) {
             if (i + k < ec) {
                 const uint2 t = e[i + k];
-                const float2 x = *reinterpret_cast<const float2 *>(v + ((size_t)t.y << (lgT + 2)));
+                const float2 x = *reinterpret_cast<const float2 *>(v + (t.y << (kLgPairTile + 2)));
                 q[k][0] = agg_step(AGG, q[k][0], __uint_as_float(t.x), x.x);
                 q[k][1] = agg_step(AGG, q[k][1], __uint_as_float(t.x), x.y);
             }
@@ -297,7 +297,7 @@ __device__ __forceinline__ float2 fold_edges_pair(const uint2 *__restrict__ e, u
 // Node p for the thread's columns; v: the thread's place in row 0.
 template <bool FAST>
 __device__ __forceinline__ void eval_node_pair(const uint4 ne, const uint2 *__restrict__ edges, char *__restrict__ v,
-                                               int p, int lgT)
+                                               int p)
 {
     const uint32_t act = ne.w & 0xffu;
     if (act == kInputAct) return;
@@ -309,13 +309,13 @@ __device__ __forceinline__ void eval_node_pair(const uint4 ne, const uint2 *__re
         f2 s;
         switch (ec) {
         case 0: s = 0ull; break;
-        case 1: s = sum_edges_pair<1>(e, v, lgT); break;
-        case 2: s = sum_edges_pair<2>(e, v, lgT); break;
-        case 3: s = sum_edges_pair<3>(e, v, lgT); break;
-        case 4: s = sum_edges_pair<4>(e, v, lgT); break;
-        case 5: s = sum_edges_pair<5>(e, v, lgT); break;
-        case 6: s = sum_edges_pair<6>(e, v, lgT); break;
-        default: s = sum_edges_pair_any(e, ec, v, lgT);
+        case 1: s = sum_edges_pair<1>(e, v); break;
+        case 2: s = sum_edges_pair<2>(e, v); break;
+        case 3: s = sum_edges_pair<3>(e, v); break;
+        case 4: s = sum_edges_pair<4>(e, v); break;
+        case 5: s = sum_edges_pair<5>(e, v); break;
+        case 6: s = sum_edges_pair<6>(e, v); break;
+        default: s = sum_edges_pair_any(e, ec, v);
         }
         a = unpack2(s);
         if (!FAST && agg == kAggMean && ec > 0) {
@@ -323,7 +323,7 @@ __device__ __forceinline__ void eval_node_pair(const uint4 ne, const uint2 *__re
             a.y = a.y / (float)ec;
         }
     } else {
-        a = agg == kAggProduct ? fold_edges_pair<kAggProduct>(e, ec, v, lgT) : fold_edges_pair<kAggMax>(e, ec, v, lgT);
+        a = agg == kAggProduct ? fold_edges_pair<kAggProduct>(e, ec, v) : fold_edges_pair<kAggMax>(e, ec, v);
         if (ec == 0) a = make_float2(0.0f, 0.0f);
     }
     const float r = __uint_as_float(ne.y), b = __uint_as_float(ne.x);
@@ -342,34 +342,29 @@ __device__ __forceinline__ void eval_node_pair(const uint4 ne, const uint2 *__re
         default: y = make_float2(z0, z1);
         }
     }
-    *reinterpret_cast<float2 *>(v + ((size_t)p << (lgT + 2))) = y;
+    *reinterpret_cast<float2 *>(v + (p << (kLgPairTile + 2))) = y;
 }
 
-// walk_levels for two columns per thread: 2^lgT columns (at least 2), of which
-// the first `cols` are asked for.
+// walk_levels for two columns per thread, of which the first `cols` are asked for.
 template <bool FAST>
-__device__ __forceinline__ void walk_pairs(const uint4 *srec, float *v, int G, int gi, int lane, int lgT, int cols)
+__device__ __forceinline__ void walk_pairs(const uint4 *srec, float *v, int G, int gi, int lane, int cols)
 {
     const uint4 h0 = srec[0], h1 = srec[1];
     const int n_levels = (int)(h0.x >> 16);
     const uint4 *nodes = srec + 2;
     const uint2 *edges = reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(srec) + h1.y);
     const uint16_t *lev = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.z);
-    const int pair = lane & ((1 << (lgT - 1)) - 1), sub = lane >> (lgT - 1), nsub = G >> (lgT - 1);
+    const int pair = lane & 31, sub = lane >> 5, nsub = G >> 5;
     char *mine = reinterpret_cast<char *>(v + 2 * pair);
     const bool ok = 2 * pair < cols;
     int p0 = (int)(h0.w >> 16);
     for (int l = 0; l < n_levels; ++l) {
         const int p1 = lev[l + 1];
         if (ok)
-            for (int p = p0 + sub; p < p1; p += nsub) {
-                if (lgT == 6) eval_node_pair<FAST>(nodes[p], edges, mine, p, 6);
-                else eval_node_pair<FAST>(nodes[p], edges, mine, p, lgT);
-            }
+            for (int p = p0 + sub; p < p1; p += nsub) eval_node_pair<FAST>(nodes[p], edges, mine, p);
         p0 = p1;
-        if (nsub > 1) group_sync(G, gi);
+        group_sync(G, gi);
     }
-    group_sync(G, gi);
 }
 
 // All non-input nodes of a staged record, for the columns this thread owns.
@@ -549,8 +544,8 @@ __device__ __forceinline__ bool run_item(const uint4 *srec, float *v, uint32_t b
         const bool col_ok = T1 || (lane & (step - 1)) < cols;
         const bool fast = (h0.w & 0xffffu) == kTraitsSumTanh;
         if constexpr (PAIRS) {
-            if (fast) walk_pairs<true>(srec, v, G, gi, lane, lgT, cols);
-            else walk_pairs<false>(srec, v, G, gi, lane, lgT, cols);
+            if (fast) walk_pairs<true>(srec, v, G, gi, lane, cols);
+            else walk_pairs<false>(srec, v, G, gi, lane, cols);
         } else if (fast) walk_levels<T1, true>(srec, v, G, gi, lane, lgT, lg_split, col_ok);
         else walk_levels<T1, false>(srec, v, G, gi, lane, lgT, lg_split, col_ok);
         for (int i = lane; i < cols * O; i += G) {
