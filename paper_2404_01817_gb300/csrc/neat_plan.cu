@@ -66,6 +66,11 @@ struct CompactPop {
 };
 
 constexpr int kCompactWarps = 4;
+// A node's edges that one lane goes through by itself; the warp shares more (2000
+// genomes of 500 inputs, 4 outputs that read them all and 300 unneeded nodes, 8
+// vectors: 146 us a step, 252 with a lane for each output's 500 edges, 165 without
+// copies).
+constexpr int kLaneEdges = 32;
 
 // Whether a header describes a record of these sizes (a plan may be created
 // before its records are written; whatever lies there then is not followed).
@@ -129,6 +134,17 @@ compact_kernel(const CompactPop *__restrict__ pops, int np, const CompactPop one
     }
     last = __reduce_max_sync(all, last);
     __syncwarp();
+    // the sources of edges i, i + step, ... below e
+    auto mark = [&](int i, int e, int step) {
+        for (; i < e; i += 4 * step) {
+            uint32_t s[4];
+#pragma unroll
+            for (int k4 = 0; k4 < 4; ++k4) s[k4] = i + k4 * step < e ? __ldg(&edges[i + k4 * step].y) : all;
+#pragma unroll
+            for (int k4 = 0; k4 < 4; ++k4)
+                if (s[k4] != all) atomicOr(bits + (s[k4] >> 5), 1u << (s[k4] & 31u));
+        }
+    };
     // from the outputs back, a round for all nodes marked since the last one:
     // a node each lane, whatever its level (rounds of one level each leave
     // most lanes idle)
@@ -147,17 +163,14 @@ compact_kernel(const CompactPop *__restrict__ pops, int np, const CompactPop one
         int k = incl - __popc(fresh);
         for (uint32_t m = fresh; m; m &= m - 1u) list[k++] = (uint16_t)(32 * lane + __ffs(m) - 1);
         __syncwarp();
-        for (int q = lane; q < count; q += 32) {
-            const uint32_t z = __ldg(&nodes[list[q]].z);
+        for (int q0 = 0; q0 < count; q0 += 32) {
+            const uint32_t z = q0 + lane < count ? __ldg(&nodes[list[q0 + lane]].z) : 0u;
             const int b = (int)(z & 0xffffu), e = b + (int)(z >> 16);
-            for (int i = b; i < e; i += 4) {
-                uint32_t s[4];
-#pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4) s[k4] = i + k4 < e ? __ldg(&edges[i + k4].y) : all;
-#pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4)
-                    if (s[k4] != all) atomicOr(bits + (s[k4] >> 5), 1u << (s[k4] & 31u));
+            for (unsigned many = __ballot_sync(all, e - b > kLaneEdges); many; many &= many - 1u) {
+                const int from = __ffs(many) - 1, wb = __shfl_sync(all, b, from), we = __shfl_sync(all, e, from);
+                mark(wb + lane, we, 32);
             }
+            if (e - b <= kLaneEdges) mark(b, e, 1);
         }
         __syncwarp();
     }
@@ -185,6 +198,18 @@ compact_kernel(const CompactPop *__restrict__ pops, int np, const CompactPop one
     auto rank = [&](uint32_t p) { return (uint32_t)(pre[p >> 5] + __popc(bits[p >> 5] & ((1u << (p & 31u)) - 1u))); };
     const uint32_t off_edge = kHeaderBytes + kNodeBytes * (uint32_t)n;
     uint2 *edges_out = reinterpret_cast<uint2 *>(dst + off_edge);
+    // edges i, i + step, ... below ec of a node whose edges begin at b, to begin at `to`
+    auto copy = [&](int b, int to, int i, int ec, int step) {
+        for (; i < ec; i += 4 * step) {
+            uint2 e[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i + q * step < ec) e[q] = __ldg(edges + b + i + q * step);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i + q * step < ec) edges_out[to + i + q * step] = make_uint2(e[q].x, rank(e[q].y));
+        }
+    };
     int carry = 0;
     unsigned lead = (unsigned)n;                               // leading positions that are inputs
     for (int k0 = 0; k0 < n; k0 += 32) {
@@ -200,18 +225,14 @@ compact_kernel(const CompactPop *__restrict__ pops, int np, const CompactPop one
         }
         const int to = carry + sum - ec;
         carry += __shfl_sync(all, sum, 31);
+        for (unsigned many = __ballot_sync(all, k < n && ec > kLaneEdges); many; many &= many - 1u) {
+            const int from = __ffs(many) - 1, wb = __shfl_sync(all, b, from), we = __shfl_sync(all, ec, from);
+            copy(wb, __shfl_sync(all, to, from), lane, we, 32);
+        }
         if (k >= n) continue;
         if ((ne.w & 0xffu) != kInputAct) lead = min(lead, (unsigned)k);
         out[2 + k] = make_uint4(ne.x, ne.y, (uint32_t)to | ((uint32_t)ec << 16), ne.w);
-        for (int i = 0; i < ec; i += 4) {
-            uint2 e[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (i + q < ec) e[q] = __ldg(edges + b + i + q);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (i + q < ec) edges_out[to + i + q] = make_uint2(e[q].x, rank(e[q].y));
-        }
+        if (ec <= kLaneEdges) copy(b, to, 0, ec, 1);
     }
     lead = __reduce_min_sync(all, lead);
     const uint32_t off_level = align16(off_edge + kEdgeBytes * (uint32_t)carry);
