@@ -1362,7 +1362,9 @@ int fill_population_bucket(const neat_pop_desc &pd, const int32_t *gidx_dev, int
                            BucketDev *out, size_t *footprint, bool own_size, int max_used, int max_rows)
 {
     const int rows = max_rows > 0 ? std::min(max_rows, pd.dims.max_nodes) : pd.dims.max_nodes;
-    const Shape sh = heuristic_shape(rows, pd.batch, block_threads);
+    // (the threads of a tile row halve below a power of two: 504 of 512 rows left
+    // do not count as fewer)
+    const Shape sh = heuristic_shape(10 * rows >= 9 * pd.dims.max_nodes ? pd.dims.max_nodes : rows, pd.batch, block_threads);
     uint32_t rec = record_max_bytes(pd.dims.num_inputs, pd.dims.num_outputs, pd.dims.max_nodes, pd.dims.max_conns);
     if (max_used > 0) rec = std::min(rec, align16((uint32_t)max_used));
     const size_t reg = ((size_t)rec + 4u * (size_t)((rows * sh.tile + 3) & ~3) + 15) & ~(size_t)15;
