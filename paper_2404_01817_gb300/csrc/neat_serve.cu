@@ -81,6 +81,27 @@ __device__ __forceinline__ void normals_of_block(uint64_t seed, int step, uint64
     out[3] = rad1 * s;
 }
 
+// Elements e .. e + 3 (e a multiple of 4) of out[n], as one store where the array
+// is aligned for it.
+template <typename T>
+__device__ __forceinline__ void store_four(T *out, uint64_t e, uint64_t n, const T v[4])
+{
+    static_assert(sizeof(T) == 4, "four words");
+    if (e + 3 >= n) {
+        for (int k = 0; k < 4; ++k)
+            if (e + k < n) out[e + k] = v[k];
+    } else if ((reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
+        uint4 w;
+        memcpy(&w, v, 16);
+        reinterpret_cast<uint4 *>(out)[e >> 2] = w;
+    } else {
+        out[e] = v[0];
+        out[e + 1] = v[1];
+        out[e + 2] = v[2];
+        out[e + 3] = v[3];
+    }
+}
+
 struct GenDesc {
     float *out;
     uint64_t count;
@@ -104,11 +125,7 @@ __global__ void gen_normals_kernel(const GenDesc *__restrict__ descs, int nd)
     if (e0 >= d.count) return;
     float z[4];
     normals_of_block(d.seed, d.step, e0 >> 2, z);
-    if (e0 + 3 < d.count && (reinterpret_cast<uintptr_t>(d.out) & 15u) == 0) {
-        reinterpret_cast<float4 *>(d.out)[e0 >> 2] = make_float4(z[0], z[1], z[2], z[3]);
-        return;
-    }
-    for (int k = 0; k < 4 && e0 + k < d.count; ++k) d.out[e0 + k] = z[k];
+    store_four(d.out, e0, d.count, z);
 }
 
 // One descriptor, passed by value.
@@ -118,11 +135,7 @@ __global__ void fill_normals_kernel(float *out, uint64_t count, uint64_t seed, i
     if (e0 >= count) return;
     float z[4];
     normals_of_block(seed, step, e0 >> 2, z);
-    if (e0 + 3 < count && (reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
-        reinterpret_cast<float4 *>(out)[e0 >> 2] = make_float4(z[0], z[1], z[2], z[3]);
-        return;
-    }
-    for (int k = 0; k < 4 && e0 + k < count; ++k) out[e0 + k] = z[k];
+    store_four(out, e0, count, z);
 }
 
 // Raw Philox words: word e = component e mod 4 of the block for counter
@@ -135,13 +148,8 @@ __global__ void gen_words_kernel(uint32_t *out, uint64_t n, uint64_t seed, uint6
         const U4 r = philox4x32_10(U4{(uint32_t)b, (uint32_t)(b >> 32), (uint32_t)stream,
                                       (uint32_t)(stream >> 32) ^ 0x574f5244u},
                                    (uint32_t)seed, (uint32_t)(seed >> 32));
-        const uint64_t e = b << 2;
-        if (e + 3 < n && (reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
-            reinterpret_cast<uint4 *>(out)[b] = make_uint4(r.x, r.y, r.z, r.w);
-        } else {
-            const uint32_t v[4] = {r.x, r.y, r.z, r.w};
-            for (uint64_t k = 0; k < 4 && e + k < n; ++k) out[e + k] = v[k];
-        }
+        const uint32_t v[4] = {r.x, r.y, r.z, r.w};
+        store_four(out, b << 2, n, v);
     }
 }
 
