@@ -209,14 +209,16 @@ __device__ __forceinline__ void eval_node_tile(const uint4 ne, const uint2 *__re
                                         : node_output(ne, agg, act, ec, a);
 }
 
-// walk_levels for several columns, from position `first` (the inputs before
-// it have their values); LGT: log2 of the tile's columns (-1: lgT).
-template <bool FAST, int LGT>
+// walk_levels for 2^lg columns, from position `first` (the inputs before it have
+// their values).  One loop for every width: beside one compiled for 32 columns, 2
+// to 4% faster there, it took 4 to 10% longer (launches of 4 and 16 vectors, 10
+// 000 genomes of 50 rows: 24.6 and 37.7 us, 26.5 and 41.6 with both; six fused
+// steps of 300 rows, 1000 genomes, 8 and 16 vectors: 94 and 130, 101 and 136).
+template <bool FAST>
 __device__ __forceinline__ void walk_tile(const uint4 *nodes, const uint2 *edges, const uint16_t *lev, float *v,
-                                          int first, int n_nodes, int n_levels, int G, int gi, int lane, int lgT,
+                                          int first, int n_nodes, int n_levels, int G, int gi, int lane, int lg,
                                           bool col_ok)
 {
-    const int lg = LGT >= 0 ? LGT : lgT;
     const int col = lane & ((1 << lg) - 1);
     const int sub = lane >> lg;
     const int nsub = G >> lg;
@@ -441,11 +443,7 @@ __device__ __forceinline__ void walk_levels(const uint4 *srec, float *v, int G, 
             group_sync(G, gi);
         }
     } else {
-        // 32 columns, the usual tile: a shift known at compile time makes a
-        // value's address one instruction
-        const int first = (int)(h0.w >> 16);
-        if (lgT == 5) walk_tile<FAST, 5>(nodes, edges, lev, v, first, n_nodes, n_levels, G, gi, lane, lgT, col_ok);
-        else walk_tile<FAST, -1>(nodes, edges, lev, v, first, n_nodes, n_levels, G, gi, lane, lgT, col_ok);
+        walk_tile<FAST>(nodes, edges, lev, v, (int)(h0.w >> 16), n_nodes, n_levels, G, gi, lane, lgT, col_ok);
     }
     group_sync(G, gi);
 }
