@@ -187,31 +187,6 @@ __device__ __forceinline__ int mask_first(uint32_t mine)
     return owner * 32 + __shfl_sync(kAll, __ffs(mine) - 1, owner);
 }
 
-// Lowest present row holding a key, for keys of any size: a slot holds the key's
-// low 24 bits and a row, and a row is taken by its whole key, as in the block
-// form's table (a malformed genome's keys at or above 2^24 are nodes of their
-// own in both).  At most half the slots are taken.
-__device__ __forceinline__ void insert_row(uint32_t *tab, uint32_t mask, int shift, const float *ns, uint32_t row)
-{
-    const uint32_t key = (uint32_t)ns[5 * row], v = (key << 8) | row;
-    for (uint32_t s = slot32(key, shift);; s = (s + 1u) & mask) {
-        const uint32_t old = atomicCAS(tab + s, kFree32, v);
-        if (old == kFree32) return;
-        if ((old >> 8) == (v >> 8) && (uint32_t)ns[5 * (old & 0xffu)] == key) {
-            atomicMin(tab + s, v);
-            return;
-        }
-    }
-}
-__device__ __forceinline__ int find_row(const uint32_t *tab, uint32_t mask, int shift, const float *ns, uint32_t key)
-{
-    for (uint32_t s = slot32(key, shift);; s = (s + 1u) & mask) {
-        const uint32_t v = tab[s];
-        if (v == kFree32) return -1;
-        if ((v >> 8) == (key & 0xffffffu) && (uint32_t)ns[5 * (v & 0xffu)] == key) return (int)(v & 0xffu);
-    }
-}
-
 struct MutWarpLayout {
     int nodes, preds, ktab, total;           // byte offsets in a warp's shared memory (connections at 0)
 };
@@ -346,10 +321,24 @@ __global__ void __launch_bounds__(128) mutate_warp_kernel(const MutArgs a)
                     for (int i = lane; i < 2 * a.Np2; i += 32) ktab[i] = kFree32;
                     for (int i = lane; i < RN * N; i += 32) preds[i] = 0u;
                     __syncwarp();
+                    // (a malformed genome's node keys beyond 24 bits do not fit the table:
+                    // its rows are searched, by the whole key as in the block form)
+                    bool wide = false;
                     for (int r = lane; r < N; r += 32)
-                        if (node_present(r)) insert_row(ktab, kmask, kshift, ns, (uint32_t)r);
-                    __syncwarp();
-                    auto row_of = [&](float k) { return find_row(ktab, kmask, kshift, ns, (uint32_t)k); };
+                        if (node_present(r)) {
+                            const uint32_t key = (uint32_t)ns[5 * r];
+                            wide |= key > 0xffffffu;
+                            insert32(ktab, kmask, kshift, key & 0xffffffu, (uint32_t)r);
+                        }
+                    wide = __any_sync(kAll, wide);
+                    __syncwarp();                        // the votes order no memory
+                    auto row_of = [&](float k) {
+                        const uint32_t key = (uint32_t)k;
+                        if (!wide) return find32(ktab, kmask, kshift, key);
+                        for (int r = 0; r < N; ++r)
+                            if (node_present(r) && (uint32_t)ns[5 * r] == key) return r;
+                        return -1;
+                    };
                     for (int c = lane; c < C; c += 32) {
                         if (!conn_present(c)) continue;
                         const int x = row_of(cs[c].x), y = row_of(cs[c].y);
