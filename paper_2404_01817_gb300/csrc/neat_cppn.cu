@@ -187,6 +187,32 @@ __device__ __forceinline__ void write_nan(float *out, const CppnArgs &a, int q0,
             out[(size_t)l * a.pairs + q] = __int_as_float(0x7fc00000);
 }
 
+// The needed nodes of a record with one level, which tells nothing of the order
+// (neat_transform_recurrent's: positions follow node rows): a warp's passes over
+// the nodes marked last (1; 2 once their sources are), until none is added.  True,
+// in some lane, when a node does not come after the nodes it reads.
+__device__ __noinline__ bool close_over_edges(uint8_t *need, const uint4 *nodes, const uint2 *packed, int n_nodes, int lane)
+{
+    bool unordered = false;
+    for (bool more = true; more;) {
+        more = false;
+        for (int p = lane; p < n_nodes; p += 32) {
+            if (need[p] != 1) continue;
+            need[p] = 2;
+            const uint32_t z = nodes[p].z;
+            for (uint32_t i = z & 0xffffu, e = i + (z >> 16); i < e; ++i) {
+                const uint32_t src = packed[i].y;
+                if (need[src] == 0) need[src] = 1;
+                unordered |= (int)src >= p && (nodes[src].w & 0xffu) != kInputAct;
+                more = true;
+            }
+        }
+        __syncwarp();
+        more = __any_sync(0xffffffffu, more);
+    }
+    return unordered;
+}
+
 template <bool WIDE>
 __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
 {
@@ -194,7 +220,7 @@ __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
     __shared__ uint64_t bar_mem;
     __shared__ float coord[256];
     __shared__ uint8_t need[kCppnMaxNodes], slot_of[kCppnMaxNodes];
-    __shared__ int failed, n_prog, unordered;
+    __shared__ int failed, n_prog;                         // n_prog: -1 where the rows are in no order to follow
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
     const int g = (int)(blockIdx.x / a.chunks);
     const int q0 = (int)(blockIdx.x - (unsigned)g * a.chunks) * a.chunk;
@@ -208,7 +234,7 @@ __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
     if (tid == 0) {
         const uint32_t bytes = min(align16(__ldg(reinterpret_cast<const uint32_t *>(grec) + 4)),
                                    (uint32_t)a.rec_words * 16u);
-        failed = unordered = 0;
+        failed = 0;
         mbar_init(bar, 1);
         mbar_arrive_expect_tx(bar, bytes);
         bulk_g2s(smem_addr(srec), grec, bytes, bar);
@@ -237,29 +263,10 @@ __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
     const uint16_t *io = reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(srec) + h1.w);
     const int p_out = io[5];
     if (tid < 32) {
-        // the nodes that the output depends on, from the last level back.  One
-        // level tells nothing of the order (neat_transform_recurrent's records:
-        // positions follow node rows): there, pass after pass over the nodes
-        // marked last (1; 2 once their sources are), until none is added, and
-        // a node must come after the nodes it reads
+        // the nodes that the output depends on, from the last level back
         if (lane == 0) need[p_out] = 1;
         __syncwarp();
-        for (bool more = n_levels == 1; more;) {
-            more = false;
-            for (int p = lane; p < n_nodes; p += 32) {
-                if (need[p] != 1) continue;
-                need[p] = 2;
-                const uint32_t z = nodes[p].z;
-                for (uint32_t i = z & 0xffffu, e = i + (z >> 16); i < e; ++i) {
-                    const uint32_t src = packed[i].y;
-                    if (need[src] == 0) need[src] = 1;
-                    if ((int)src >= p && (nodes[src].w & 0xffu) != kInputAct) unordered = 1;
-                    more = true;
-                }
-            }
-            __syncwarp();
-            more = __any_sync(0xffffffffu, more);
-        }
+        const bool unordered = n_levels == 1 && close_over_edges(need, nodes, packed, n_nodes, lane);
         for (int l = n_levels - 1; l > 0; --l) {
             for (int p = lev[l] + lane; p < lev[l + 1]; p += 32)
                 if (need[p]) {
@@ -282,15 +289,16 @@ __global__ void __launch_bounds__(kCppnThreads) cppn_kernel(const CppnArgs a)
             }
             count += __popc(m);
         }
-        if (lane == 0) n_prog = count;
+        const unsigned none = __ballot_sync(0xffffffffu, unordered);
+        if (lane == 0) n_prog = none ? -1 : count;
     }
     __syncthreads();
-    if (unordered) {
+    const int np = n_prog;
+    if (np < 0) {
         write_nan(out, a, q0, qend);
         return;
     }
     // four columns per thread, as many threads as the rows leave room for
-    const int np = n_prog;
     const int active = min(nt, (a.tile_bytes / (16 * (5 + np))) & ~31);
     const int row = 16 * active;                           // bytes of a tile row
     // sources become byte offsets of their rows (a node that is not evaluated
