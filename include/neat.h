@@ -733,7 +733,8 @@ NEAT_API int neat_forward_multi_noalloc(const neat_pop_desc *pops_host, int32_t 
  * Queued requests are admitted, in arrival order (a later one that fits may
  * pass one that does not), as pool memory frees up; their genome tensors are
  * copied in and transformed once, then copied without the nodes that no output
- * depends on into the memory of the genome tensors, where that is large enough.
+ * depends on into the memory of the genome tensors, where that is large enough and
+ * the request has steps enough to pay for it.
  * Every scheduler tick advances each active
  * request by one step -- one kernel generating the step's observations, one
  * persistent-kernel launch evaluating all active requests together -- so

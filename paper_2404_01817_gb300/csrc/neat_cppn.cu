@@ -26,7 +26,8 @@
 // Bound by issue (66% of the slots at 22 warps per SM): the edges' shared
 // memory reads, the dispatches and the transcendentals; the only traffic is 4
 // bytes written per weight.  1000 genomes (up to 32 nodes, 96 connections), 3
-// layers of 16 x 16: 0.36 ms and 0.23 G warp instructions, 1.45 TB/s written.
+// layers of 16 x 16: 0.33 to 0.38 ms by population, the benchmark's 0.41 (perf/
+// cases.py seed 5: 0.36 ms and 0.23 G warp instructions, 1.45 TB/s written).
 // One pair per thread and column, every node, every block evaluated: 2.70 ms
 // and 3.07 G; four columns and one evaluation per pair, without the list of
 // needed nodes and with a fixed 128 threads: 1.29 ms and 0.75 G at 12 warps.

@@ -481,8 +481,12 @@ extern "C" int neat_forward_ex(const void *transformed_dev, int32_t pop, neat_di
     // place, 48 staged; 1000 / 4000: 43 and 67).  Below, the staged copy's one
     // long read beats the walk's many short ones (300 genomes: 21 us in place,
     // 13 staged)
-    const long staged = 152L * (long)(227u * 1024u / ((size_t)a.rec_words * 16 + (size_t)a.val_floats * 4 + 1024u));
-    if (!launch_host && batch == 1 && a.rec_copy_bytes == 0 && 2L * pop > 5L * std::max(1L, staged)) {
+    const auto waves_of_staged = [&]() {
+        const DeviceCaps caps = device_caps();
+        const long fit = caps.smem_per_sm / (long)((size_t)a.rec_words * 16 + (size_t)a.val_floats * 4 + 1024u);
+        return (double)pop / std::max(1L, caps.sms * fit);
+    };
+    if (!launch_host && batch == 1 && a.rec_copy_bytes == 0 && waves_of_staged() > 2.5) {
         const size_t smem = 4u * (size_t)a.val_floats * kDirectWarps;
         rc = allow_dynamic_smem(reinterpret_cast<const void *>(forward_direct_kernel), smem, "forward: shared memory per block");
         if (rc) return rc;

@@ -470,8 +470,8 @@ struct AlwaysFits {
 // tile, walks the levels and writes the outputs.
 //   xb: inputs of the item [bt][I]; yb: its outputs [bt][O]; vcap: floats of
 //   the value tile, at least one column of the genome's nodes (a genome with
-//   more nodes than the tile has rows takes fewer columns at a time; WHOLE: it
-//   has the rows, all columns at once).
+//   more nodes than the tile has rows takes fewer columns at a time; WHOLE: the
+//   tile has the rows, all columns at once, vcap is not read).
 //   fits(bytes of the record, values of its columns): asked once the record is
 //   there; where it is false, run_item returns false with nothing evaluated.
 // PAIRS: two columns per thread (tile 64, WHOLE).

@@ -140,7 +140,9 @@ __device__ unsigned int g_lanes_error;
 // Bound by issue (72% of the slots).  10 000 Ant-sized genomes: 34 us, against
 // 54 us for heights by levels with shared-memory atomics and ready tests that
 // walked every node's edges in every beat; without the unneeded fifth of the
-// nodes a step of the compiled programs takes 3.42 us instead of 3.65.
+// nodes a step of 10 000 random Ant-sized networks in perf/cases.py takes 3.42 us
+// instead of 3.65 (the benchmark's population, whose deepest networks need all
+// their nodes: 3.68 and 3.65).
 // Writes the genome's schedule into the scratch and its sort key into
 // meas[g] = beats | max lane quads << 8 | flags << 24.  Thread 0 of block 0
 // also writes the buffer header (its reductions zero).
@@ -816,7 +818,7 @@ __device__ __forceinline__ void load_beat_head(BeatState &st, uint4 ne, uint32_t
 
 // A lone warp counts a run's beats; warps that share it step to its end (the
 // counted form for both: 10 000 recurrent genomes of 20 nodes 8.5 -> 9.6 us a
-// step; the stepped form for both: the Ant step 3.67 -> 3.72 us).
+// step; the stepped form for both: the benchmark's Ant step 3.67 -> 3.72 us).
 template <int W, typename F>
 __device__ __forceinline__ void each_beat(const F &beat, int &b, int len, int end)
 {

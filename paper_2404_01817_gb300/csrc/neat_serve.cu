@@ -322,7 +322,7 @@ bool copies_pay(const neat_request &r)
 // depends on, evaluated from then on.  They take the place of the genome
 // tensors, where these are large enough; how large the copies are comes back
 // without waiting for it, and until it has, the launch shapes allow for any.
-// A burst of 24 requests of 20 steps: 9.1 ms against 11.4 without the copies.
+// A burst of 24 requests of 20 steps: 8.4 ms against 10.6 without the copies.
 int compact_request(neat_server *S, Request *R)
 {
     const neat_request &r = R->r;
